@@ -1,12 +1,12 @@
 // Section 2 pixel selection and weak-field fallback, Section 5.5 seeds and
 // polarity, and the order-preserving selection of the pixels to invert.
+#include "async_copy.cuh"
 #include "kernels.h"
 
 namespace genesis {
 
 namespace {
 
-constexpr int kClassifyBlock = 128;  // four pixels (one warp each) per block
 constexpr int kSelectTile = 2048;    // flags per selection tile
 constexpr int kSelectBlock = 256;    // threads per selection block, 8 flags each
 constexpr double kPi = 3.14159265358979323846;
@@ -17,13 +17,6 @@ constexpr double kPi = 3.14159265358979323846;
 // start at zero; concurrent calls share it and therefore race.
 static __device__ __align__(256) int g_select_tiles[(ME_SELECT_STATIC_MAX_PIX + kSelectTile - 1) / kSelectTile];
 
-// One pixel's Stokes rows as FP64 values.
-template <class RO> struct Rows {
-    const RO *o;
-    int nl;
-    __device__ __forceinline__ double at(int s, int j) const { return (double)o[s * nl + j]; }
-};
-
 // Three-point parabola vertex through (x0, y0), (x1, y1), (x2, y2), without
 // contraction; x1 when the points are collinear.
 __device__ __forceinline__ double vertex3(double x0, double x1, double x2, double y0, double y1, double y2)
@@ -33,17 +26,6 @@ __device__ __forceinline__ double vertex3(double x0, double x1, double x2, doubl
     const double num = __dsub_rn(__dmul_rn(__dmul_rn(d0, d0), e2), __dmul_rn(__dmul_rn(d2, d2), e0));
     const double den = __dsub_rn(__dmul_rn(d0, e2), __dmul_rn(d2, e0));
     return den != 0.0 ? __dsub_rn(x1, __ddiv_rn(__dmul_rn(0.5, num), den)) : x1;
-}
-
-// Three-point second difference of Stokes row s at interior point c on the
-// (possibly non-uniform) grid.
-template <class RO>
-__device__ __forceinline__ double second_diff(const double *lam, const Rows<RO> &r, int s, int c)
-{
-    const double h1 = __dsub_rn(lam[c], lam[c - 1]), h2 = __dsub_rn(lam[c + 1], lam[c]);
-    const double y0 = r.at(s, c - 1), y1 = r.at(s, c), y2 = r.at(s, c + 1);
-    const double num = __dmul_rn(2.0, __dsub_rn(__dmul_rn(h1, __dsub_rn(y2, y1)), __dmul_rn(h2, __dsub_rn(y1, y0))));
-    return __ddiv_rn(num, __dmul_rn(__dmul_rn(h1, h2), __dadd_rn(h1, h2)));
 }
 
 // Trapezoid weight of point j in the window [lo, hi].
@@ -59,157 +41,299 @@ __device__ __forceinline__ double degrees(double rad) { return __ddiv_rn(__dmul_
 
 // A seed (B, psi, chi) from B_par and B_perp, psi reflected into the pixel's
 // polarity half.
-__device__ __forceinline__ void put_seed(double *sd, double bpar, double bperp, double chi, int pol)
+__device__ __forceinline__ void put_seed(double *sd, double bpar, double bperp, double psi, double chi, int pol)
 {
-    double psi = degrees(atan2(bperp, bpar));
     if ((pol > 0 && psi > 90.0) || (pol < 0 && psi < 90.0)) psi = __dsub_rn(180.0, psi);
     sd[0] = __dsqrt_rn(__dadd_rn(__dmul_rn(bpar, bpar), __dmul_rn(bperp, bperp)));
     sd[1] = psi;
     sd[2] = chi;
 }
 
-// Warp argmin (want_max = false) or argmax of v with ties to the lowest index.
-__device__ __forceinline__ void warp_arg(double &v, int &i, bool want_max)
+// An integer in the order of the finite doubles (-0 and +0 equal): FP64
+// comparisons take the FP64 pipe, integer ones do not.
+__device__ __forceinline__ long long order64(double x)
 {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double ov = __shfl_xor_sync(0xffffffffu, v, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, i, off);
-        const bool better = want_max ? (ov > v) : (ov < v);
-        if (better || (ov == v && oi < i)) {
-            v = ov;
-            i = oi;
-        }
-    }
+    const long long b = __double_as_longlong(x);
+    return b == (long long)0x8000000000000000ull ? 0 : b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-// Section 2 threshold, weak-field estimate, polarity and seeds: one warp per
-// pixel, FP64 throughout.  Extrema are lane-parallel (exact); each running
-// sum is taken by one lane in increasing index, so every result except the
-// angles (atan2) repeats the plain sequential evaluation bit for bit.
+__device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_of(double x) { return fabs(x); }
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
+
+// Exact FP32 -> FP64 widening of normal numbers with integer operations (the
+// conversion instruction takes the FP64 pipe).
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+    if (m - 0x00800000u >= 0x7f000000u) return (double)x;  // zero, subnormal, infinity, NaN
+    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// Correctly rounded a / b for a divisor whose correctly rounded reciprocal rb
+// is at hand (Markstein 1990): two quotient corrections by exact remainders,
+// five FP64 operations where the division takes 8 to 9.  rb = 0 marks a
+// divisor outside 2^+-200; those, and dividends outside 2^+-700 other than 0,
+// are divided outright (no remainder may underflow).
+__device__ __forceinline__ double div_known(double a, double b, double rb)
+{
+    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
+    const bool zero = (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) == 0u;
+    if (rb == 0.0 || !(zero || ea - 323u < 1400u)) return __ddiv_rn(a, b);
+    double q = __dmul_rn(a, rb);
+    q = __fma_rn(__fma_rn(-b, q, a), rb, q);
+    return __fma_rn(__fma_rn(-b, q, a), rb, q);
+}
+__device__ __forceinline__ double known_rcp(double b)
+{
+    const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+    return eb - 823u < 400u ? __ddiv_rn(1.0, b) : 0.0;
+}
+
+constexpr int kChunk = 32;            // wavelengths staged at once
+constexpr int kPitch = kChunk + 1;    // tile row pitch: a column read touches 32 banks
+
+// Stage wavelengths [j0, j0 + kChunk) of the warp's 32 pixels: t[s][pixel]
+// [j - j0], rows beyond the map repeating its last pixel.
 template <class RO>
-__global__ void __launch_bounds__(kClassifyBlock)
-k_classify(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, int npix, const KClassify c)
+__device__ __forceinline__ void stage_chunk(RO *t, const RO *obs, int nl, int pix0, int npix, int j0)
 {
     const int lane = threadIdx.x & 31;
-    const int pix = blockIdx.x * (kClassifyBlock / 32) + (threadIdx.x >> 5);
-    if (pix >= npix) return;
-    const int nl = pb.n_lambda;
+    __syncwarp();  // the tile's readers are done
+    if (j0 + lane < nl) {
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) {
+            const RO *o = obs + (size_t)min(pix0 + r, npix - 1) * 4 * nl + j0 + lane;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) copy_async(t + (s * 32 + r) * kPitch + lane, o + (size_t)s * nl);
+        }
+    }
+    copy_wait();
+}
+
+// Wavelength-only factors of the sums, the same for every pixel: h = lam[j+1]
+// - lam[j], the second difference's denominator h1 h2 (h1 + h2) at j, their
+// reciprocals (known_rcp), and the trapezoid weight of j in the line window.
+struct GridTables {
+    double h, rh, den, rden, wt;
+};
+
+// What the two warps of a ROLES = 2 block tell each other, per pixel.
+struct ClassifyExchange {
+    double qa, ub, dd, tvi, tvd;  // from the first
+    int ip, im, pol;              // from the second
+};
+
+// Section 2 threshold, weak-field estimate, polarity and seeds in FP64, one
+// pixel per lane.  Each running sum is taken in increasing index, so every
+// result except the angles (atan2) repeats the plain sequential evaluation
+// bit for bit.  Bound by the FP64 pipe, which takes 16 clocks of an SM per
+// warp instruction whether one lane or all 32 are active: with a warp per
+// pixel (its sums on 15 lanes, six divergent groups) an instruction served
+// one pixel, here it serves 32.  The lanes read their pixels' columns of a
+// tile that the warp stages 32 wavelengths at a time (rows of 128 bytes, so
+// HBM reads stay coalesced; pitch 33, so the column reads are conflict-free).
+// Extrema of the observed values are compared in their own type and those of
+// I +- V as integers, off the FP64 pipe.  262 144 two-line pixels of a float
+// cube: 48.5 ms with a warp per pixel, 1.29 ms
+// with a lane.
+// One warp per block, so that the blocks spread evenly over the SMs.  ROLES =
+// 2 gives a block's 32 pixels a second warp that takes the sums of V, L and
+// the centres of gravity: at one warp to an SM partition the chain of dependent
+// FP64 operations is the time, and this shortens it (64 pixels: 104 -> 68 us).
+template <class RO, int ROLES>
+__global__ void __launch_bounds__(ROLES * 32)
+k_classify(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, int npix, const KClassify c)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int nl = pb.n_lambda, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool role_a = ROLES == 1 || warp == 0, role_b = ROLES == 1 || warp == 1;
     const double *lam = pb.lam;
-    const Rows<RO> r{obs + (size_t)pix * 4 * nl, nl};
     const int lo = c.c_lo, hi = c.c_hi;
-
-    // extrema: |Q|, |U|, |V| over the grid; the I+V, I-V cores and the V
-    // lobes over the line window
-    double qx = 0.0, ux = 0.0, vx = 0.0;
-    for (int j = lane; j < nl; j += 32) {
-        qx = fmax(qx, fabs(r.at(1, j)));
-        ux = fmax(ux, fabs(r.at(2, j)));
-        vx = fmax(vx, fabs(r.at(3, j)));
+    GridTables *tab = (GridTables *)smem;
+    RO *t = (RO *)(tab + nl) + warp * 4 * 32 * kPitch;
+    for (int j = max(lo - 1, 0) + threadIdx.x; j <= min(hi + 1, nl - 1); j += blockDim.x) {
+        GridTables g = {};
+        if (j + 1 < nl) {
+            g.h = __dsub_rn(lam[j + 1], lam[j]);
+            g.rh = known_rcp(g.h);
+            if (j > 0) {
+                const double h1 = __dsub_rn(lam[j], lam[j - 1]);
+                g.den = __dmul_rn(__dmul_rn(h1, g.h), __dadd_rn(h1, g.h));
+                g.rden = known_rcp(g.den);
+            }
+        }
+        if (j >= lo && j <= hi) g.wt = trap_w(lam, lo, hi, j);
+        tab[j] = g;
     }
-    double vp = INFINITY, vm = INFINITY, vhi = -INFINITY, vlo = INFINITY;
+    __syncthreads();
+    const int pix0 = blockIdx.x * 32;
+    const int pix = pix0 + lane;
+    const RO *col = t + lane * kPitch;  // this lane's pixel, Stokes s at col[s * 32 * kPitch]
+    constexpr int S = 32 * kPitch;
+    int staged = -1;
+    auto stage = [&](int j0) {
+        if (staged != j0) stage_chunk(t, obs, nl, pix0, npix, j0);
+        staged = j0;
+    };
+
+    // quiet-window means of I, Q, U, V and variances of Q, U, V
+    const double nq = (double)(c.q_hi - c.q_lo);
+    double mean[4] = {0.0, 0.0, 0.0, 0.0}, var[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int j0 = c.q_lo / kChunk * kChunk; j0 < c.q_hi; j0 += kChunk) {
+        stage(j0);
+        for (int j = max(j0, c.q_lo); j < min(j0 + kChunk, c.q_hi); ++j)
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (role_a || s == 0) mean[s] = __dadd_rn(mean[s], widen(col[s * S + j - j0]));
+    }
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+        if (role_a || s == 0) mean[s] = __ddiv_rn(mean[s], nq);
+    if (role_a) {
+        for (int j0 = c.q_lo / kChunk * kChunk; j0 < c.q_hi; j0 += kChunk) {
+            stage(j0);
+            for (int j = max(j0, c.q_lo); j < min(j0 + kChunk, c.q_hi); ++j)
+#pragma unroll
+                for (int s = 1; s < 4; ++s) {
+                    const double d = __dsub_rn(widen(col[s * S + j - j0]), mean[s]);
+                    var[s] = __dadd_rn(var[s], __dmul_rn(d, d));
+                }
+        }
+#pragma unroll
+        for (int s = 1; s < 4; ++s) var[s] = __ddiv_rn(var[s], nq);
+    }
+    const double ic = mean[0];
+
+    // one pass over the grid: extrema of |Q|, |U|, |V|; in the line window the
+    // I+V, I-V cores, the V lobes and the sums
+    RO qx = 0, ux = 0, vx = 0, vhi = 0, vlo = 0;
+    long long vp = 0, vm = 0;
     int ip = hi + 1, im = hi + 1, jhi = hi + 1, jlo = hi + 1;
-    for (int j = lo + lane; j <= hi; j += 32) {
-        const double I = r.at(0, j), V = r.at(3, j);
-        const double a = __dadd_rn(I, V), b = __dsub_rn(I, V);
-        if (a < vp) { vp = a; ip = j; }
-        if (b < vm) { vm = b; im = j; }
-        if (V > vhi) { vhi = V; jhi = j; }
-        if (V < vlo) { vlo = V; jlo = j; }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        qx = fmax(qx, __shfl_xor_sync(0xffffffffu, qx, off));
-        ux = fmax(ux, __shfl_xor_sync(0xffffffffu, ux, off));
-        vx = fmax(vx, __shfl_xor_sync(0xffffffffu, vx, off));
-    }
-    warp_arg(vp, ip, false);
-    warp_arg(vm, im, false);
-    warp_arg(vhi, jhi, true);
-    warp_arg(vlo, jlo, false);
-
-    // sequential sums, one per lane
-    const int nq = c.q_hi - c.q_lo;
-    double acc = 0.0, acc2 = 0.0;
-    if (lane < 4) {  // quiet-window mean (and, for Q, U, V, variance)
-        for (int j = c.q_lo; j < c.q_hi; ++j) acc = __dadd_rn(acc, r.at(lane, j));
-        acc = __ddiv_rn(acc, (double)nq);
-        if (lane > 0) {
-            for (int j = c.q_lo; j < c.q_hi; ++j) {
-                const double d = __dsub_rn(r.at(lane, j), acc);
-                acc2 = __dadd_rn(acc2, __dmul_rn(d, d));
+    double qa = 0.0, ub = 0.0, dd = 0.0;    // least-squares sums of Q I'', U I'', I''^2
+    double av = 0.0, al = 0.0;              // trapezoid integrals of |V| and L
+    double tvi = 0.0, tvd = 0.0;            // total variation of I and I'
+    double np = 0.0, dp = 0.0, nm = 0.0, dm = 0.0;  // centre-of-gravity moments of I_c - (I +- V)
+    double y1 = 0.0, q1 = 0.0, u1 = 0.0;  // I, Q, U at j-1
+    double e1 = 0.0, sl1 = 0.0;           // I[j-1] - I[j-2] and its slope
+    for (int j0 = 0; j0 < nl; j0 += kChunk) {
+        const int j1 = min(j0 + kChunk, nl);
+        if (!role_a && (j1 <= lo || j0 > hi)) continue;  // only the line window matters to the second role
+        stage(j0);
+        for (int j = j0; j < j1; ++j) {
+            const RO qr = col[S + j - j0], ur = col[2 * S + j - j0], vr = col[3 * S + j - j0];
+            if (role_a) {
+                qx = max_of(qx, abs_of(qr));
+                ux = max_of(ux, abs_of(ur));
+                vx = max_of(vx, abs_of(vr));
             }
-            acc2 = __ddiv_rn(acc2, (double)nq);
-        }
-    } else if (lane < 7) {  // least-squares sums of Q I'', U I'', I''^2
-        for (int j = lo > 1 ? lo : 1; j <= hi && j + 1 < nl; ++j) {
-            const double d2 = second_diff(lam, r, 0, j);
-            const double y = lane == 6 ? d2 : r.at(lane - 3, j);
-            acc = __dadd_rn(acc, __dmul_rn(y, d2));
-        }
-    } else if (lane < 9) {  // trapezoid integrals of |V| and L
-        for (int j = lo; j <= hi; ++j) {
-            const double wj = trap_w(lam, lo, hi, j);
-            double y;
-            if (lane == 7) {
-                y = fabs(r.at(3, j));
-            } else {
-                const double q = r.at(1, j), u = r.at(2, j);
-                y = __dsqrt_rn(__dadd_rn(__dmul_rn(q, q), __dmul_rn(u, u)));
+            if (j + 2 < lo || j > hi + 1) continue;
+            const double I = widen(col[j - j0]), Q = widen(qr), U = widen(ur);
+            if (role_a) {
+                const double e = __dsub_rn(I, y1);
+                const int m = j - 1;  // the point whose neighbours are now known
+                if (m >= lo && m >= 1 && m <= hi) {
+                    const double h1 = tab[m - 1].h, h2 = tab[m].h;
+                    const double num = __dsub_rn(__dmul_rn(h1, e), __dmul_rn(h2, e1));
+                    const double d2 = div_known(__dadd_rn(num, num), tab[m].den, tab[m].rden);
+                    qa = __dadd_rn(qa, __dmul_rn(q1, d2));
+                    ub = __dadd_rn(ub, __dmul_rn(u1, d2));
+                    dd = __dadd_rn(dd, __dmul_rn(d2, d2));
+                }
+                if (m >= lo && j <= hi) {
+                    tvi = __dadd_rn(tvi, fabs(e));
+                    const double sl = div_known(e, tab[m].h, tab[m].rh);
+                    if (m > lo) tvd = __dadd_rn(tvd, fabs(__dsub_rn(sl, sl1)));
+                    sl1 = sl;
+                }
+                y1 = I;
+                q1 = Q;
+                u1 = U;
+                e1 = e;
             }
-            acc = __dadd_rn(acc, __dmul_rn(wj, y));
-        }
-    } else if (lane == 9) {  // total variation of I
-        for (int j = lo; j < hi; ++j) acc = __dadd_rn(acc, fabs(__dsub_rn(r.at(0, j + 1), r.at(0, j))));
-    } else if (lane == 10) {  // total variation of I'
-        for (int j = lo + 1; j < hi; ++j) {
-            const double sl = __ddiv_rn(__dsub_rn(r.at(0, j + 1), r.at(0, j)), __dsub_rn(lam[j + 1], lam[j]));
-            const double sr = __ddiv_rn(__dsub_rn(r.at(0, j), r.at(0, j - 1)), __dsub_rn(lam[j], lam[j - 1]));
-            acc = __dadd_rn(acc, fabs(__dsub_rn(sl, sr)));
-        }
-    }
-    const double ic = __shfl_sync(0xffffffffu, acc, 0);
-    if (lane >= 11 && lane < 15) {  // centre-of-gravity moments of I_c - (I +- V)
-        const bool plus = lane < 13, moment = (lane & 1) != 0;
-        for (int j = lo; j <= hi; ++j) {
-            const double wj = trap_w(lam, lo, hi, j);
-            const double I = r.at(0, j), V = r.at(3, j);
-            const double a = __dmul_rn(wj, __dsub_rn(ic, plus ? __dadd_rn(I, V) : __dsub_rn(I, V)));
-            acc = __dadd_rn(acc, moment ? __dmul_rn(a, lam[j]) : a);
+            if (role_b && j >= lo && j <= hi) {
+                const double V = widen(vr), wt = tab[j].wt, lj = lam[j];
+                const double a = __dadd_rn(I, V), b = __dsub_rn(I, V);
+                const long long ka = order64(a), kb = order64(b);
+                if (j == lo || ka < vp) { vp = ka; ip = j; }
+                if (j == lo || kb < vm) { vm = kb; im = j; }
+                if (j == lo || vr > vhi) { vhi = vr; jhi = j; }
+                if (j == lo || vr < vlo) { vlo = vr; jlo = j; }
+                av = __dadd_rn(av, __dmul_rn(wt, fabs(V)));
+                al = __dadd_rn(al, __dmul_rn(wt, __dsqrt_rn(__dadd_rn(__dmul_rn(Q, Q), __dmul_rn(U, U)))));
+                const double ga = __dmul_rn(wt, __dsub_rn(ic, a)), gb = __dmul_rn(wt, __dsub_rn(ic, b));
+                np = __dadd_rn(np, __dmul_rn(ga, lj));
+                dp = __dadd_rn(dp, ga);
+                nm = __dadd_rn(nm, __dmul_rn(gb, lj));
+                dm = __dadd_rn(dm, gb);
+            }
         }
     }
-    double v[16], v2[4];
-#pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = __shfl_sync(0xffffffffu, acc, q);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) v2[q] = __shfl_sync(0xffffffffu, acc2, q);
-    if (lane != 0) return;
-
-    // threshold
-    const double p = __ddiv_rn(
-        __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(qx, qx), __dmul_rn(ux, ux)), __dmul_rn(vx, vx))), ic);
-    const double sp = __ddiv_rn(__dmul_rn(c.p_thresh, __dsqrt_rn(__dadd_rn(__dadd_rn(v2[1], v2[2]), v2[3]))), ic);
-    const int flag = p > sp ? 1 : 0;
-    const int pol = jhi < jlo ? 1 : (jhi > jlo ? -1 : 0);
+    int pol = jhi < jlo ? 1 : (jhi > jlo ? -1 : 0);
+    if (ROLES == 2) {
+        __shared__ ClassifyExchange s_x[32];
+        ClassifyExchange &x = s_x[lane];
+        if (role_a) {
+            x.qa = qa;
+            x.ub = ub;
+            x.dd = dd;
+            x.tvi = tvi;
+            x.tvd = tvd;
+        } else {
+            x.ip = ip;
+            x.im = im;
+            x.pol = pol;
+        }
+        __syncthreads();
+        qa = x.qa;
+        ub = x.ub;
+        dd = x.dd;
+        tvi = x.tvi;
+        tvd = x.tvd;
+        ip = x.ip;
+        im = x.im;
+        pol = x.pol;
+    }
+    if (pix >= npix) return;
+    const RO *o = obs + (size_t)pix * 4 * nl;
 
     // weak field
-    auto core = [&](int bi, bool plus) {
-        if (bi - 1 < 0 || bi + 1 >= nl) return lam[bi];
-        double y[3];
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            const double I = r.at(0, bi - 1 + t), V = r.at(3, bi - 1 + t);
-            y[t] = plus ? __dadd_rn(I, V) : __dsub_rn(I, V);
-        }
-        return vertex3(lam[bi - 1], lam[bi], lam[bi + 1], y[0], y[1], y[2]);
-    };
     const double two_kz = __dmul_rn(2.0, c.kz);
-    const double bpar = __ddiv_rn(__dsub_rn(core(ip, true), core(im, false)), two_kz);
-    const double qa = v[4], ub = v[5], dd = v[6];
     double chi = degrees(__dmul_rn(0.5, atan2(-ub, -qa)));
     if (chi < 0.0) chi = __dadd_rn(chi, 180.0);
     const double amp = __dsqrt_rn(__dadd_rn(__dmul_rn(qa, qa), __dmul_rn(ub, ub)));
     const double bperp = dd > 0.0 ? __ddiv_rn(__dsqrt_rn(__ddiv_rn(__dmul_rn(4.0, amp), dd)), c.kz) : 0.0;
+    double *sd = c.seeds ? c.seeds + (size_t)pix * 12 : nullptr;
+    if (role_b && sd) {
+        const double bpi = tvi > 0.0 ? __ddiv_rn(__dmul_rn(pol < 0 ? -1.0 : 1.0, av), __dmul_rn(c.kz, tvi)) : 0.0;
+        const double bti = tvd > 0.0 ? __ddiv_rn(__dsqrt_rn(__ddiv_rn(__dmul_rn(4.0, al), tvd)), c.kz) : 0.0;
+        put_seed(sd + 3, bpi, bti, degrees(atan2(bti, bpi)), chi, pol);
+        const double bcog =
+            (dp != 0.0 && dm != 0.0) ? __ddiv_rn(__dsub_rn(__ddiv_rn(np, dp), __ddiv_rn(nm, dm)), two_kz) : 0.0;
+        put_seed(sd + 6, bcog, bperp, degrees(atan2(bperp, bcog)), chi, pol);
+    }
+    if (!role_a) return;
+
+    // threshold
+    const double qd = (double)qx, ud = (double)ux, vd = (double)vx;
+    const double p = __ddiv_rn(
+        __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(qd, qd), __dmul_rn(ud, ud)), __dmul_rn(vd, vd))), ic);
+    const double sp = __ddiv_rn(__dmul_rn(c.p_thresh, __dsqrt_rn(__dadd_rn(__dadd_rn(var[1], var[2]), var[3]))), ic);
+    const int flag = p > sp ? 1 : 0;
+
+    auto core = [&](int bi, bool plus) {
+        if (bi - 1 < 0 || bi + 1 >= nl) return lam[bi];
+        double y[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double I = (double)o[bi - 1 + k], V = (double)o[3 * nl + bi - 1 + k];
+            y[k] = plus ? __dadd_rn(I, V) : __dsub_rn(I, V);
+        }
+        return vertex3(lam[bi - 1], lam[bi], lam[bi + 1], y[0], y[1], y[2]);
+    };
+    const double bpar = __ddiv_rn(__dsub_rn(core(ip, true), core(im, false)), two_kz);
     const double bmag = __dsqrt_rn(__dadd_rn(__dmul_rn(bpar, bpar), __dmul_rn(bperp, bperp)));
     const double theta = degrees(atan2(bperp, bpar));
 
@@ -227,18 +351,9 @@ k_classify(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, int 
         wo[3] = bpar;
         wo[4] = bperp;
     }
-    if (c.seeds) {
-        double *sd = c.seeds + (size_t)pix * 12;
-        put_seed(sd, bpar, bperp, chi, pol);
-        const double av = v[7], al = v[8], tvi = v[9], tvd = v[10];
-        const double bpi = tvi > 0.0 ? __ddiv_rn(__dmul_rn(pol < 0 ? -1.0 : 1.0, av), __dmul_rn(c.kz, tvi)) : 0.0;
-        const double bti = tvd > 0.0 ? __ddiv_rn(__dsqrt_rn(__ddiv_rn(__dmul_rn(4.0, al), tvd)), c.kz) : 0.0;
-        put_seed(sd + 3, bpi, bti, chi, pol);
-        const double np = v[11], dp = v[12], nm = v[13], dm = v[14];
-        const double bcog =
-            (dp != 0.0 && dm != 0.0) ? __ddiv_rn(__dsub_rn(__ddiv_rn(np, dp), __ddiv_rn(nm, dm)), two_kz) : 0.0;
-        put_seed(sd + 6, bcog, bperp, chi, pol);
-        put_seed(sd + 9, bpar, bperp, chi, pol);
+    if (sd) {
+        put_seed(sd, bpar, bperp, theta, chi, pol);
+        put_seed(sd + 9, bpar, bperp, theta, chi, pol);
         sd[9] = 0.0;
     }
     if (c.best && !flag) {  // weak-field answer for the pixels below the threshold
@@ -373,17 +488,30 @@ cudaError_t launch_prefit_bounds(const double *p_hat, int npix, const KPrefitBou
     return cudaGetLastError();
 }
 
+namespace {
+
+template <class RO, int ROLES>
+cudaError_t classify_t(const KProblem &pb, const void *obs, int npix, const KClassify &c, cudaStream_t st)
+{
+    const int smem = pb.n_lambda * (int)sizeof(GridTables) + ROLES * 4 * 32 * kPitch * (int)sizeof(RO);
+    auto kern = k_classify<RO, ROLES>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(npix + 31) / 32, 32 * ROLES, smem, st>>>(pb, (const RO *)obs, npix, c);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// The second role pays while two warps for every 32 pixels are at most one to
+// each of the 608 SM partitions; beyond that the FP64 pipe is the limit.
 cudaError_t launch_classify(const KProblem &pb, int dtype, const void *obs, int npix, const KClassify &c,
                             cudaStream_t st)
 {
     if (npix <= 0) return cudaSuccess;
-    const int per = kClassifyBlock / 32;
-    const int grid = (npix + per - 1) / per;
-    if (dtype == ME_F32)
-        k_classify<float><<<grid, kClassifyBlock, 0, st>>>(pb, (const float *)obs, npix, c);
-    else
-        k_classify<double><<<grid, kClassifyBlock, 0, st>>>(pb, (const double *)obs, npix, c);
-    return cudaGetLastError();
+    const bool chain = npix <= 152 * 4 / 2 * 32;
+    if (dtype == ME_F32) return chain ? classify_t<float, 2>(pb, obs, npix, c, st) : classify_t<float, 1>(pb, obs, npix, c, st);
+    return chain ? classify_t<double, 2>(pb, obs, npix, c, st) : classify_t<double, 1>(pb, obs, npix, c, st);
 }
 
 cudaError_t select_static_scratch(void **ptr, size_t *bytes)

@@ -1,4 +1,5 @@
 // Stokes synthesis, Jacobian, adjoint and FP64 chi-square kernels (sm_103a).
+#include "async_copy.cuh"
 #include "kernels.h"
 #include "me_jac.cuh"
 #include "rng_device.cuh"
@@ -261,38 +262,148 @@ k_chi2_f64(const __grid_constant__ KProblem pb, const RO *__restrict__ obs,
     }
 }
 
-// Section 5.1 centre of symmetry, one warp per pixel: lanes scan candidates,
-// each sums |I(i+j) - I(i-j)| in FP64 in increasing j; warp argmin (ties to
-// the lowest index); lane 0 refines with the three-point parabola vertex,
-// written without contraction.
-template <class RO>
-__global__ void __launch_bounds__(kSynthBlock)
+// One pixel's search of k_line_centre on its staged row I (index 0 = grid
+// point 0): T is the type its sums are exact or rounded in.
+__device__ __forceinline__ double abs_add(double s, double a, double b) { return __dadd_rn(s, fabs(__dsub_rn(a, b))); }
+__device__ __forceinline__ long long abs_add(long long s, long long a, long long b)
+{
+    const long long d = a - b;
+    return s + (d < 0 ? -d : d);
+}
+constexpr long long kNoSum = 0x7fffffffffffffffll;  // above every sum
+// Sums are >= 0, so an FP64 sum's bits order it; NaN is never the least.
+__device__ __forceinline__ long long sum_order(double s) { return s == s ? __double_as_longlong(s) : kNoSum; }
+__device__ __forceinline__ long long sum_order(long long s) { return s; }
+
+// On return best = the least sum, bi its index (0x7fffffff: none) on every
+// lane of the pixel, y0 and y2 the sums at bi - 1 and bi + 1 on its first lane
+// where both are candidates.
+template <int G, class T>
+__device__ __forceinline__ void centre_search(const T *I, int W, int lo, int hi, int sub, T &best, int &bi, T &y0, T &y2)
+{
+    auto S = [&](int i) {
+        T s = T(0);
+        for (int j = 1; j <= W; ++j) s = abs_add(s, I[i + j], I[i - j]);
+        return s;
+    };
+    long long key = kNoSum;
+    best = T(0);
+    bi = 0x7fffffff;
+    for (int i = lo + sub; i <= hi; i += G) {
+        const T s = S(i);
+        if (sum_order(s) < key) {
+            key = sum_order(s);
+            best = s;
+            bi = i;
+        }
+    }
+#pragma unroll
+    for (int off = G / 2; off > 0; off >>= 1) {
+        const long long ok = __shfl_xor_sync(0xffffffffu, key, off);
+        const T os = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+        if (ok < key || (ok == key && oi < bi)) {
+            key = ok;
+            best = os;
+            bi = oi;
+        }
+    }
+    const bool inner = bi != 0x7fffffff && bi - 1 >= lo && bi + 1 <= hi;
+    y0 = y2 = T(0);
+    if (G == 1) {
+        if (inner) {
+            y0 = S(bi - 1);
+            y2 = S(bi + 1);
+        }
+    } else {  // one on each of two lanes
+        if (inner && sub < 2) y0 = S(bi + 2 * sub - 1);
+        y2 = __shfl_down_sync(0xffffffffu, y0, 1);
+    }
+}
+
+// Section 5.1 centre of symmetry, G lanes per pixel, 32 / G pixels per warp:
+// S_i = sum_j |I(i+j) - I(i-j)| in FP64 in increasing j, candidates i dealt to
+// the pixel's lanes, the argmin over i (ties to the lowest index) and the
+// three-point parabola vertex, written without contraction.
+// In FP64 the sums would bind the kernel: the FP64 pipe takes 16 clocks of an
+// SM per warp instruction (whether one lane or 32 are active, so a warp per
+// pixel wastes it on ragged rounds).  A float cube's samples are multiples of
+// 2^(emin - 150), emin the row's least biased exponent, so where the row's
+// exponents span few enough octaves that 24 bits, a sign, the span and the W
+// terms fit 53 bits, every difference and sum is exact in FP64 and equals the
+// same sum of 64-bit integers, which run on the integer pipe; other rows (and
+// double cubes) are summed in FP64.  262 144 pixels, W = 10, 33 candidates:
+// 2.40 ms with a warp per pixel in FP64, 0.47 ms with these lanes in FP64,
+// 0.15 ms with the integer sums.
+template <class RO, int G>
+__global__ void __launch_bounds__(32)
 k_line_centre(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, int npix, int W, int lo,
               int hi, double *__restrict__ lam_c, int *__restrict__ idx)
 {
-    const int lane = threadIdx.x & 31;
-    const int pix = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (pix >= npix) return;
-    const int nl = pb.n_lambda;
-    const RO *I = obs + (size_t)pix * 4 * nl;
-    auto S = [&](int i) {
-        double s = 0.0;
-        for (int j = 1; j <= W; ++j) s = __dadd_rn(s, fabs(__dsub_rn((double)I[i + j], (double)I[i - j])));
-        return s;
-    };
-    double best = INFINITY;
+    extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int PIX = 32 / G;
+    const int lane = threadIdx.x, nl = pb.n_lambda, sub = lane % G;
+    const int pix0 = blockIdx.x * PIX, pix = pix0 + lane / G;
+    double y0 = 0.0, y1 = 0.0, y2 = 0.0;
     int bi = 0x7fffffff;
-    for (int i = lo + lane; i <= hi; i += 32) {
-        const double s = S(i);
-        if (s < best || (s == best && i < bi)) { best = s; bi = i; }
+    if (lo <= hi) {
+        // I over [lo - W, hi + W], an odd row pitch (conflict-free column reads)
+        const int j0 = lo - W, span = hi + W - j0 + 1, pitch = span | 1;
+        bool exact = sizeof(RO) == 4;
+        if constexpr (sizeof(RO) == 4) {
+            long long *t = (long long *)smem;
+            const unsigned room = 28 - (32 - __clz(W - 1));  // octaves left beside 25 bits and the terms' carry
+            unsigned e_mine = 1u;
+            float *raw = (float *)(t + PIX * pitch);  // the rows as they are
+            for (int r = 0; r < PIX; ++r) {
+                const float *o = obs + (size_t)min(pix0 + r, npix - 1) * 4 * nl + j0;
+                for (int j = lane; j < span; j += 32) copy_async(raw + r * pitch + j, o + j);
+            }
+            copy_wait();
+            for (int r = 0; r < PIX && exact; ++r) {
+                const float *o = raw + r * pitch;
+                unsigned emin = 255u, emax = 1u;
+                for (int j = lane; j < span; j += 32) {
+                    const unsigned m = __float_as_uint(o[j]) & 0x7fffffffu;
+                    const unsigned e = max(m >> 23, 1u);
+                    if (m) emin = min(emin, e);
+                    emax = max(emax, e);
+                }
+                emin = __reduce_min_sync(0xffffffffu, emin);
+                emax = __reduce_max_sync(0xffffffffu, emax);
+                exact = emax < 255u && (emin == 255u || emax - emin <= room);
+                emin = min(emin, 254u);  // an all-zero row
+                if (r == lane / G) e_mine = emin;
+                for (int j = lane; j < span; j += 32) {
+                    const unsigned b = __float_as_uint(o[j]), e = (b >> 23) & 0xffu;
+                    const unsigned mant = (b & 0x7fffffu) | (e ? 0x800000u : 0u);
+                    const long long v = mant ? (long long)mant << min(max(e, 1u) - emin, 63u) : 0;
+                    t[r * pitch + j] = (int)b < 0 ? -v : v;
+                }
+            }
+            if (exact) {
+                __syncwarp();
+                long long s1, s0, s2;
+                centre_search<G>(t + (lane / G) * pitch - j0, W, lo, hi, sub, s1, bi, s0, s2);
+                const double unit = __hiloint2double((int)((e_mine + 873u) << 20), 0);  // 2^(emin - 150)
+                y0 = (double)s0 * unit;
+                y1 = (double)s1 * unit;
+                y2 = (double)s2 * unit;
+            }
+        }
+        if (!exact) {
+            double *t = (double *)smem;
+            __syncwarp();
+#pragma unroll 8
+            for (int r = 0; r < PIX; ++r) {
+                const RO *o = obs + (size_t)min(pix0 + r, npix - 1) * 4 * nl + j0;
+                for (int j = lane; j < span; j += 32) t[r * pitch + j] = (double)o[j];
+            }
+            __syncwarp();
+            centre_search<G>(t + (lane / G) * pitch - j0, W, lo, hi, sub, y1, bi, y0, y2);
+        }
     }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const double os = __shfl_xor_sync(0xffffffffu, best, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (os < best || (os == best && oi < bi)) { best = os; bi = oi; }
-    }
-    if (lane != 0) return;
+    if (pix >= npix || sub != 0) return;
     if (bi == 0x7fffffff) {
         lam_c[pix] = NAN;
         if (idx) idx[pix] = -1;
@@ -301,7 +412,6 @@ k_line_centre(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, i
     double xc = pb.lam[bi];
     if (bi - 1 >= lo && bi + 1 <= hi) {
         const double x0 = pb.lam[bi - 1], x1 = pb.lam[bi], x2 = pb.lam[bi + 1];
-        const double y0 = S(bi - 1), y1 = best, y2 = S(bi + 1);
         const double d0 = __dsub_rn(x1, x0), d2 = __dsub_rn(x1, x2);
         const double e0 = __dsub_rn(y1, y0), e2 = __dsub_rn(y1, y2);
         const double num = __dsub_rn(__dmul_rn(__dmul_rn(d0, d0), e2), __dmul_rn(__dmul_rn(d2, d2), e0));
@@ -395,18 +505,43 @@ cudaError_t launch_vjp(const KProblem &pb, int dtype, const double *params, cons
     return vjp_t<double, 0>(pb, params, mu_px, n, gs, gp, st);
 }
 
+namespace {
+
+template <class RO, int G>
+cudaError_t line_centre_t(const KProblem &pb, const void *obs, int npix, int W, int lo, int hi, double *lam_c,
+                          int *idx, cudaStream_t st)
+{
+    constexpr int PIX = 32 / G;
+    const int smem = lo <= hi ? PIX * ((hi - lo + 2 * W + 1) | 1) * (sizeof(RO) == 4 ? 12 : 8) : 0;
+    auto kern = k_line_centre<RO, G>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(npix + PIX - 1) / PIX, 32, smem, st>>>(pb, (const RO *)obs, npix, W, lo, hi, lam_c, idx);
+    return cudaGetLastError();
+}
+
+// Lanes per pixel: as many as leave at most one warp to each of the 608 SM
+// partitions, whose FP64 pipe one warp's chain of dependent adds already
+// fills; then the shortest chain is the fastest.  Beyond that, one.
+template <class RO>
+cudaError_t line_centre_r(const KProblem &pb, const void *obs, int npix, int W, int lo, int hi, double *lam_c,
+                          int *idx, cudaStream_t st)
+{
+    const int warps = 152 * 4;
+    if (npix <= warps) return line_centre_t<RO, 32>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    if (npix <= 4 * warps) return line_centre_t<RO, 8>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    if (npix <= 16 * warps) return line_centre_t<RO, 2>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    return line_centre_t<RO, 1>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+}
+
+}  // namespace
+
 cudaError_t launch_line_centre(const KProblem &pb, int dtype, const void *obs, int npix, int W, int lo,
                                int hi, double *lam_c, int *idx, cudaStream_t st)
 {
     if (npix <= 0) return cudaSuccess;
-    const int per = kSynthBlock / 32;
-    if (dtype == ME_F32)
-        k_line_centre<float><<<(npix + per - 1) / per, kSynthBlock, 0, st>>>(pb, (const float *)obs, npix, W, lo,
-                                                                            hi, lam_c, idx);
-    else
-        k_line_centre<double><<<(npix + per - 1) / per, kSynthBlock, 0, st>>>(pb, (const double *)obs, npix, W,
-                                                                             lo, hi, lam_c, idx);
-    return cudaGetLastError();
+    return dtype == ME_F32 ? line_centre_r<float>(pb, obs, npix, W, lo, hi, lam_c, idx, st)
+                           : line_centre_r<double>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
 }
 
 cudaError_t launch_chi2_f64(const KProblem &pb, int dtype, const void *obs, const double *w,
