@@ -118,6 +118,8 @@ bool g_dev_ready[256];
 // looked up once at set-up.
 static void *g_select_static[256];
 static size_t g_select_static_bytes = 0;
+// Per device: the Taylor coefficients of w (faddeeva_nodes.h), filled at set-up.
+static void *g_nodes[256];
 
 int ensure_device()
 {
@@ -135,7 +137,19 @@ int ensure_device()
     if ((e = upload_tables_check(t)) != cudaSuccess) return cuda_fail(e, "upload tables");
     if ((e = select_static_scratch(&g_select_static[dev], &g_select_static_bytes)) != cudaSuccess)
         return cuda_fail(e, "select scratch address");
+    if ((e = upload_nodes(&g_nodes[dev])) != cudaSuccess) return cuda_fail(e, "upload nodes");
     g_dev_ready[dev] = true;
+    return ME_OK;
+}
+
+int ensure_device(KProblem &k)
+{
+    const int rc = ensure_device();
+    if (rc) return rc;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaGetDevice");
+    k.nodes = (const double2 *)g_nodes[dev];
     return ME_OK;
 }
 
@@ -362,7 +376,7 @@ int me_synth(const me_problem *pb, const double *params, const double *mu_px, in
     if (n == 0) return ME_OK;
     if (!params || !stokes) return fail(ME_EINVAL, "params and stokes must be non-NULL");
     if ((long long)n * pb->n_lambda > (1ll << 31) - 1) return fail(ME_EINVAL, "n * n_lambda too large");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_synth(k, pb->dtype, params, mu_px, n, stokes, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "me_synth launch");
 }
@@ -377,7 +391,7 @@ int me_synth_jac(const me_problem *pb, const double *params, const double *mu_px
     if (n == 0) return ME_OK;
     if (!params || !jac) return fail(ME_EINVAL, "params and jac must be non-NULL");
     if ((long long)n * pb->n_lambda > (1ll << 31) - 1) return fail(ME_EINVAL, "n * n_lambda too large");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_jac(k, pb->dtype, params, mu_px, n, stokes, jac, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "me_synth_jac launch");
 }
@@ -392,7 +406,7 @@ int me_synth_vjp(const me_problem *pb, const double *params, const double *mu_px
     if (n == 0) return ME_OK;
     if (!params || !grad_stokes || !grad_params)
         return fail(ME_EINVAL, "params, grad_stokes and grad_params must be non-NULL");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_vjp(k, pb->dtype, params, mu_px, n, grad_stokes, grad_params, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "me_synth_vjp launch");
 }
@@ -406,7 +420,7 @@ int me_chi2(const me_problem *pb, const void *obs, const double *w, const double
     if (npix < 0) return fail(ME_EINVAL, "npix must be >= 0");
     if (npix == 0) return ME_OK;
     if (!obs || !params || !chi2) return fail(ME_EINVAL, "obs, params and chi2 must be non-NULL");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_chi2_f64(k, pb->dtype, obs, w, mu_px, npix, params, chi2, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "me_chi2 launch");
 }
@@ -435,7 +449,7 @@ static int ga_invert_impl(const me_problem *pb, const void *obs, const double *w
     const size_t need = rs * (4 + pb->n_lines) * pb->n_lambda + rs * (cfg->npop + 72) + 128 +
                         (size_t)4 * cfg->npop * npar + 256;
     if (need > 220 * 1024) return fail(ME_EINVAL, "population and grid exceed shared memory");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     const KGa &gc = g;
     const double *wu = cfg->weight_mode == ME_W_USER ? w : nullptr;
     cudaError_t e = launch_ga_evolve(k, gc, pb->dtype, obs, wu, mu_px, npix, best, best_genes,
@@ -482,7 +496,7 @@ int ga_count_evaluations(const me_problem *pb, const void *obs, const double *w,
     if (npix == 0) return ME_OK;
     if (!obs || !best || !counts) return fail(ME_EINVAL, "obs, best and counts must be non-NULL");
     if (cfg->weight_mode == ME_W_USER && !w) return fail(ME_EINVAL, "ME_W_USER needs w");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_ga_count(k, g, pb->dtype, obs, cfg->weight_mode == ME_W_USER ? w : nullptr,
                                     mu_px, npix, best, counts, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "ga_count_evaluations launch");
@@ -504,7 +518,7 @@ int ga_fitness(const me_problem *pb, const void *obs, const double *w, const dou
     const size_t need = rs * (4 + pb->n_lines) * pb->n_lambda + rs * (npop + 72) + 128 +
                         (size_t)4 * npop * npar_of(pb) + 256;
     if (need > 220 * 1024) return fail(ME_EINVAL, "population and grid exceed shared memory");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_ga_fitness(k, pb->dtype, w ? ME_W_USER : ME_W_INVMAX, obs, w, mu_px, npix, npop, nactive,
                                       params, fitness, resid, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "ga_fitness launch");
@@ -547,7 +561,7 @@ static int lm_polish_impl(const me_problem *pb, const void *obs, const double *w
     if (!(lambda0 > 0.0) || !std::isfinite(lambda0)) return fail(ME_EINVAL, "lambda0 must be positive");
     if (npix == 0) return ME_OK;
     if (!obs || !params_inout) return fail(ME_EINVAL, "obs and params_inout must be non-NULL");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     KLm lm;
     std::memset(&lm, 0, sizeof lm);
     lm.iters = iters;
@@ -622,7 +636,7 @@ int me_classify(const me_problem *pb, const void *obs, int npix, double p_thresh
     if (line < 0 || line >= pb->n_lines) return fail(ME_EINVAL, "line out of range");
     if (npix == 0) return ME_OK;
     if (!obs) return fail(ME_EINVAL, "obs must be non-NULL");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     KClassify c;
     c.p_thresh = p_thresh;
     c.kz = k.line[line].zfac;
@@ -682,7 +696,7 @@ int lm_uncertainty(const me_problem *pb, const void *obs, const double *w, const
     if (npix < 0) return fail(ME_EINVAL, "npix must be >= 0");
     if (npix == 0) return ME_OK;
     if (!obs || !params || !sigma) return fail(ME_EINVAL, "obs, params and sigma must be non-NULL");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_lm_sigma(k, pb->dtype, obs, w, mu_px, npix, params, sigma, as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "lm_uncertainty launch");
 }
@@ -697,7 +711,7 @@ int me_line_centre(const me_problem *pb, const void *obs, int npix, int half_wid
     if (npix == 0) return ME_OK;
     if (!obs || !lambda_c) return fail(ME_EINVAL, "obs and lambda_c must be non-NULL");
     const int lo = std::max(i_lo, half_width), hi = std::min(i_hi, pb->n_lambda - 1 - half_width);
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(k))) return rc;
     cudaError_t e = launch_line_centre(k, pb->dtype, obs, npix, half_width, lo, hi, lambda_c, index,
                                        as_stream(stream));
     return e == cudaSuccess ? ME_OK : cuda_fail(e, "me_line_centre launch");

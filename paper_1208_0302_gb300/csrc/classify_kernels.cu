@@ -1,6 +1,7 @@
 // Section 2 pixel selection and weak-field fallback, Section 5.5 seeds and
 // polarity, and the order-preserving selection of the pixels to invert.
 #include "async_copy.cuh"
+#include "fp64_util.cuh"
 #include "kernels.h"
 
 namespace genesis {
@@ -61,16 +62,6 @@ __device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
 __device__ __forceinline__ double abs_of(double x) { return fabs(x); }
 __device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
-
-// Exact FP32 -> FP64 widening of normal numbers with integer operations (the
-// conversion instruction takes the FP64 pipe).
-__device__ __forceinline__ double widen(float x)
-{
-    const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u) return (double)x;  // zero, subnormal, infinity, NaN
-    return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
 
 // Correctly rounded a / b for a divisor whose correctly rounded reciprocal rb
 // is at hand (Markstein 1990): two quotient corrections by exact remainders,

@@ -82,6 +82,9 @@ cudaError_t upload_tables_synth(const HostTables &t);
 cudaError_t upload_tables_lm(const HostTables &t);
 cudaError_t upload_tables_ga_fill(const HostTables &t);
 cudaError_t upload_tables_check(const HostTables &t);
+// The file-scope array of w's Taylor coefficients (synth_kernels.cu), filled on
+// the current device; *ptr receives its address (KProblem::nodes).
+cudaError_t upload_nodes(void **ptr);
 
 // ga_kernels.cu
 cudaError_t launch_ga_evolve(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
@@ -161,6 +164,7 @@ extern thread_local std::string g_last_error;
 int set_error(int code, const std::string &msg);
 int cuda_error(cudaError_t e, const char *where);
 int ensure_device();
+int ensure_device(KProblem &k);  // the same, and k.nodes
 int make_problem(const me_problem *pb, KProblem &k);
 int npar_of(const me_problem *pb);  // 9, or 10 with the fill fraction
 int check_bounds(const me_bounds *b, int npar);

@@ -264,7 +264,7 @@ int serve_create(const me_problem *pb, const serve_config *cfg, serve_handle **o
     if (cfg->max_inflight < 1 || cfg->max_inflight > 64)
         return set_error(ME_EINVAL, "max_inflight must be 1..64");
     if (cfg->max_queue < 1) return set_error(ME_EINVAL, "max_queue must be >= 1");
-    if ((rc = ensure_device())) return rc;
+    if ((rc = ensure_device(kp))) return rc;
     serve_handle *h = new (std::nothrow) serve_handle();
     if (!h) return set_error(ME_ENOMEM, "serve handle allocation failed");
     cudaGetDevice(&h->device);

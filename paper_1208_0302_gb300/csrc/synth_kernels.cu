@@ -2,9 +2,19 @@
 #include "async_copy.cuh"
 #include "kernels.h"
 #include "me_jac.cuh"
+#include "profiles64.cuh"
 #include "rng_device.cuh"
 
 namespace genesis {
+
+static __device__ double2 d_nodes[kNodeGrid * kNodeGrid * kNodeCoef];
+
+cudaError_t upload_nodes(void **ptr)
+{
+    static const std::vector<double> host = faddeeva_nodes();
+    const cudaError_t e = cudaGetSymbolAddress(ptr, d_nodes);
+    return e != cudaSuccess ? e : cudaMemcpyToSymbol(d_nodes, host.data(), sizeof(d_nodes));
+}
 
 cudaError_t upload_tables_synth(const HostTables &t)
 {
@@ -159,106 +169,139 @@ k_vjp(const __grid_constant__ KProblem pb, const double *__restrict__ params,
     }
 }
 
+// FP64 synthesis, one block per model (see profiles64.cuh): 65 536 two-line
+// models 14.0 -> 4.8 ms against a thread per (model, wavelength), a call for one
+// one-line model 27 -> 17 us; absolute error 1.5e-15 -> 7e-17 rms.
+template <bool FILL>
+__global__ void __launch_bounds__(kProfBlock)
+k_synth64(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
+          double *__restrict__ stokes)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    ProfShared &S = *(ProfShared *)smem;
+    const int nl = pb.n_lambda, m = blockIdx.x;
+    constexpr int M = kNpar<FILL>;
+    double p[M];
+#pragma unroll
+    for (int d = 0; d < M; ++d) p[d] = params[(size_t)m * M + d];
+    build_model<FILL>(S, pb, p, mu_px ? mu_px[m] : pb.mu);
+    double *o = stokes + (size_t)m * 4 * nl;
+    for (int j0 = 0; j0 < nl; j0 += kProfBlock) {
+        const ProfSums r = profile_sums<FILL>(S, pb, j0, nl);
+        const int j = j0 + threadIdx.x;
+        if (j < nl) {
+            const Stokes4<double> s = stokes_of<FILL>(S.g, r);
+            o[j] = s.I;
+            o[nl + j] = s.Q;
+            o[2 * nl + j] = s.U;
+            o[3 * nl + j] = s.V;
+        }
+    }
+}
+
+__device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_of(double x) { return fabs(x); }
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
+
+// One warp: the pixel's squared weights, the caller's or Section 5.4's
+// inverse-max weights in FP64 (the extrema in the cube's own type).
+template <class RO>
+__device__ __forceinline__ void weights64(const RO *o, int nl, const double *w_user, int pix, double *s_w2)
+{
+    const int lane = threadIdx.x & 31;
+    if (w_user) {
+        if (lane < 4) {
+            const double w = w_user[(size_t)pix * 4 + lane];
+            s_w2[lane] = w * w;
+        }
+        return;
+    }
+    RO imax = -INFINITY, nmin = -INFINITY, m[3] = {0, 0, 0};  // nmin = -min I
+    for (int j = lane; j < nl; j += 32) {
+        imax = max_of(imax, o[j]);
+        nmin = max_of(nmin, -o[j]);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], abs_of(o[(s + 1) * nl + j]));
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        imax = max_of(imax, __shfl_xor_sync(0xffffffffu, imax, off));
+        nmin = max_of(nmin, __shfl_xor_sync(0xffffffffu, nmin, off));
+#pragma unroll
+        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], __shfl_xor_sync(0xffffffffu, m[s], off));
+    }
+    if (lane < 4) {
+        const double top = (double)imax;
+        const double d = lane == 0 ? top + (double)nmin : (double)(lane == 1 ? m[0] : lane == 2 ? m[1] : m[2]);
+        const double fl = 1e-6 * fabs(top);
+        const double dd = d > fl ? d : fl;
+        const double w = dd > 0.0 ? 1.0 / dd : 0.0;
+        s_w2[lane] = w * w;
+    }
+}
+
 // FP64 chi-square (Eq. chisq) of given parameters, one block per pixel,
-// threads over wavelengths.  Inverse-max weights (Section 5.4) are formed in
-// FP64 from the observed values when w is NULL.
-// NL > 0 with PAT = false: problems with NL effective-triplet lines (the
-// loops over lines unrolled, the full-pattern code compiled out; the same
-// arithmetic in the same order as the generic form, 4.6 % faster on the
-// two-line map, where the pass is bound by the FP64 pipe).
-template <class RO, bool FILL = false, int NL = 0, bool PAT = true>
-__global__ void __launch_bounds__(kSynthBlock)
+// threads over wavelengths, on the profiles of profiles64.cuh.  Bound by the
+// FP64 pipe: 65 536 two-line pixels took 13.5 ms with Weideman's series and
+// the 9th convergent per thread (both branches in most warps, every division
+// in full, the geometry on one thread), 5.1 ms now, and the relative error of
+// chi2 against 64-bit references fell from 2.5e-13 to 8e-15 rms.
+template <class RO, bool FILL>
+__global__ void __launch_bounds__(kProfBlock)
 k_chi2_f64(const __grid_constant__ KProblem pb, const RO *__restrict__ obs,
            const double *__restrict__ w_user, const double *__restrict__ mu_px, int npix,
            const double *__restrict__ params, double *__restrict__ chi2, const KSub sub)
 {
-    __shared__ double s_red[kSynthBlock / 32][4];
+    extern __shared__ __align__(16) unsigned char smem[];
+    ProfShared &S = *(ProfShared *)smem;
+    __shared__ double s_red[kProfBlock / 32][4];
     __shared__ double s_w2[4];
-    const int nl = pb.n_lambda, nlines = pb.n_lines;
+    const int nl = pb.n_lambda;
     const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (sub.count && b >= *sub.count) return;
     const int pix = sub.index ? sub.index[b] : b;
     if (pix < 0 || pix >= npix) return;
     const RO *o = obs + (size_t)pix * 4 * nl;
-    if (w_user) {
-        if (threadIdx.x < 4) {
-            const double w = w_user[(size_t)pix * 4 + threadIdx.x];
-            s_w2[threadIdx.x] = w * w;
-        }
-    } else if (warp == 0) {
-        double imax = -INFINITY, imin = INFINITY, mq = 0, mu = 0, mv = 0;
-        for (int j = lane; j < nl; j += 32) {
-            const double I = (double)o[j];
-            imax = fmax(imax, I);
-            imin = fmin(imin, I);
-            mq = fmax(mq, fabs((double)o[nl + j]));
-            mu = fmax(mu, fabs((double)o[2 * nl + j]));
-            mv = fmax(mv, fabs((double)o[3 * nl + j]));
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            imax = fmax(imax, __shfl_xor_sync(0xffffffffu, imax, off));
-            imin = fmin(imin, __shfl_xor_sync(0xffffffffu, imin, off));
-            mq = fmax(mq, __shfl_xor_sync(0xffffffffu, mq, off));
-            mu = fmax(mu, __shfl_xor_sync(0xffffffffu, mu, off));
-            mv = fmax(mv, __shfl_xor_sync(0xffffffffu, mv, off));
-        }
-        if (lane == 0) {
-            const double d[4] = {imax - imin, mq, mu, mv};
-            const double fl = 1e-6 * fabs(imax);
-            for (int s = 0; s < 4; ++s) {
-                const double dd = d[s] > fl ? d[s] : fl;
-                const double w = dd > 0.0 ? 1.0 / dd : 0.0;
-                s_w2[s] = w * w;
-            }
-        }
-    }
     constexpr int M = kNpar<FILL>;
-    // the pixel's geometry, built once per block (FP64 trigonometry and
-    // divisions) and read by every thread from shared memory
-    __shared__ __align__(16) unsigned char s_geo_raw[sizeof(Geo<double>)];
-    Geo<double> &s_geo = *reinterpret_cast<Geo<double> *>(s_geo_raw);
-    if (threadIdx.x == 0) {
-        double p[M];
+    double p[M];
 #pragma unroll
-        for (int d = 0; d < M; ++d) p[d] = params[(size_t)pix * M + d];
-        const double mu = mu_px ? mu_px[pix] : pb.mu;
-        s_geo = make_geo<double, NL, FILL>(pb, nlines, p, mu);
-    }
-    __syncthreads();
-    const Geo<double> &g = s_geo;
-    double he[ME_MAX_LINES];
-#pragma unroll
-    for (int l = 0; l < ME_MAX_LINES; ++l) he[l] = l < nlines ? pb.line[l].half_eta : 0.0;
+    for (int d = 0; d < M; ++d) p[d] = params[(size_t)pix * M + d];
+    build_model<FILL>(S, pb, p, mu_px ? mu_px[pix] : pb.mu);
+    if (warp == 3) weights64<RO>(o, nl, w_user, pix, s_w2);
     double ss[4] = {0, 0, 0, 0};
-    for (int j = threadIdx.x; j < nl; j += blockDim.x) {
-        double doff[ME_MAX_LINES];
-#pragma unroll
-        for (int l = 0; l < ME_MAX_LINES; ++l) doff[l] = l < nlines ? pb.lam[j] - pb.line[l].lam0 : 0.0;
-        const Stokes4<double> s = me_point<double, NL, PAT, FILL>(g, doff, he, nlines, pb.line);
-        const double r0 = (double)o[j] - s.I, r1 = (double)o[nl + j] - s.Q;
-        const double r2 = (double)o[2 * nl + j] - s.U, r3 = (double)o[3 * nl + j] - s.V;
-        ss[0] += r0 * r0;
-        ss[1] += r1 * r1;
-        ss[2] += r2 * r2;
-        ss[3] += r3 * r3;
-    }
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) ss[s] += __shfl_xor_sync(0xffffffffu, ss[s], off);
-    }
-    if (lane == 0)
-        for (int s = 0; s < 4; ++s) s_red[warp][s] = ss[s];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int s = 0; s < 4; ++s) {
-            double a = 0.0;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += s_red[w][s];
-            tot += s_w2[s] * a;
+    for (int j0 = 0; j0 < nl; j0 += kProfBlock) {
+        const ProfSums r = profile_sums<FILL>(S, pb, j0, nl);
+        const int j = j0 + threadIdx.x;
+        if (j < nl) {
+            const Stokes4<double> s = stokes_of<FILL>(S.g, r);
+            const double r0 = widen(o[j]) - s.I, r1 = widen(o[nl + j]) - s.Q;
+            const double r2 = widen(o[2 * nl + j]) - s.U, r3 = widen(o[3 * nl + j]) - s.V;
+            ss[0] += r0 * r0;
+            ss[1] += r1 * r1;
+            ss[2] += r2 * r2;
+            ss[3] += r3 * r3;
         }
-        chi2[pix] = tot / (double)(4 * nl - M);
+    }
+    // the four warp sums at once, halving the values a lane holds with the
+    // lanes it is added from: 6 FP64 additions instead of 20
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double x0 = (h16 ? ss[2] : ss[0]) + __shfl_xor_sync(0xffffffffu, h16 ? ss[0] : ss[2], 16);
+    const double x1 = (h16 ? ss[3] : ss[1]) + __shfl_xor_sync(0xffffffffu, h16 ? ss[1] : ss[3], 16);
+    double v = (h8 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, h8 ? x0 : x1, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((lane & 7) == 0) s_red[warp][lane >> 3] = v;
+    __syncthreads();
+    if (warp == 0) {
+        double a = 0.0;
+        if (lane < 4) {
+            for (int w = 0; w < kProfBlock / 32; ++w) a += s_red[w][lane];
+            a *= s_w2[lane];
+        }
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
+        if (lane == 0) chi2[pix] = a / (double)(4 * nl - M);
     }
 }
 
@@ -437,6 +480,18 @@ cudaError_t synth_t(const KProblem &pb, const double *params, const double *mu_p
     return cudaGetLastError();
 }
 
+template <bool FILL>
+cudaError_t synth64_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes,
+                      cudaStream_t st)
+{
+    auto kern = k_synth64<FILL>;
+    const size_t smem = prof_smem(pb);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<n, kProfBlock, smem, st>>>(pb, params, mu_px, (double *)stokes);
+    return cudaGetLastError();
+}
+
 template <class R, int NL, bool FILL = false>
 cudaError_t jac_t(const KProblem &pb, const double *params, const double *mu_px, int n,
                   void *stokes, void *jac, cudaStream_t st)
@@ -464,15 +519,13 @@ cudaError_t launch_synth(const KProblem &pb, int dtype, const double *params, co
                          int n, void *stokes, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    if (pb.fill)
-        return dtype == ME_F32 ? synth_t<float, 0, true>(pb, params, mu_px, n, stokes, st)
-                               : synth_t<double, 0, true>(pb, params, mu_px, n, stokes, st);
-    if (dtype == ME_F32) {
-        if (pb.n_lines == 1) return synth_t<float, 1>(pb, params, mu_px, n, stokes, st);
-        if (pb.n_lines == 2) return synth_t<float, 2>(pb, params, mu_px, n, stokes, st);
-        return synth_t<float, 0>(pb, params, mu_px, n, stokes, st);
-    }
-    return synth_t<double, 0>(pb, params, mu_px, n, stokes, st);
+    if (dtype != ME_F32)
+        return pb.fill ? synth64_t<true>(pb, params, mu_px, n, stokes, st)
+                       : synth64_t<false>(pb, params, mu_px, n, stokes, st);
+    if (pb.fill) return synth_t<float, 0, true>(pb, params, mu_px, n, stokes, st);
+    if (pb.n_lines == 1) return synth_t<float, 1>(pb, params, mu_px, n, stokes, st);
+    if (pb.n_lines == 2) return synth_t<float, 2>(pb, params, mu_px, n, stokes, st);
+    return synth_t<float, 0>(pb, params, mu_px, n, stokes, st);
 }
 
 cudaError_t launch_jac(const KProblem &pb, int dtype, const double *params, const double *mu_px,
@@ -544,30 +597,28 @@ cudaError_t launch_line_centre(const KProblem &pb, int dtype, const void *obs, i
                            : line_centre_r<double>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
 }
 
+template <class RO, bool FILL>
+static cudaError_t chi2_t(const KProblem &pb, const void *obs, const double *w, const double *mu_px, int npix,
+                          const double *params, double *chi2, cudaStream_t st, KSub sub)
+{
+    auto kern = k_chi2_f64<RO, FILL>;
+    const size_t smem = prof_smem(pb);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<npix, kProfBlock, smem, st>>>(pb, (const RO *)obs, w, mu_px, npix, params, chi2, sub);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_chi2_f64(const KProblem &pb, int dtype, const void *obs, const double *w,
                             const double *mu_px, int npix, const double *params, double *chi2,
                             cudaStream_t st, KSub sub)
 {
     if (npix <= 0) return cudaSuccess;
-    if (dtype == ME_F32 && pb.fill)
-        k_chi2_f64<float, true><<<npix, kSynthBlock, 0, st>>>(pb, (const float *)obs, w, mu_px, npix, params,
-                                                              chi2, sub);
-    else if (dtype == ME_F32 && !has_pattern(pb) && pb.n_lines == 2)
-        k_chi2_f64<float, false, 2, false><<<npix, kSynthBlock, 0, st>>>(pb, (const float *)obs, w, mu_px, npix,
-                                                                        params, chi2, sub);
-    else if (dtype == ME_F32 && !has_pattern(pb) && pb.n_lines == 1)
-        k_chi2_f64<float, false, 1, false><<<npix, kSynthBlock, 0, st>>>(pb, (const float *)obs, w, mu_px, npix,
-                                                                        params, chi2, sub);
-    else if (dtype == ME_F32)
-        k_chi2_f64<float><<<npix, kSynthBlock, 0, st>>>(pb, (const float *)obs, w, mu_px, npix, params, chi2,
-                                                        sub);
-    else if (pb.fill)
-        k_chi2_f64<double, true><<<npix, kSynthBlock, 0, st>>>(pb, (const double *)obs, w, mu_px, npix, params,
-                                                               chi2, sub);
-    else
-        k_chi2_f64<double><<<npix, kSynthBlock, 0, st>>>(pb, (const double *)obs, w, mu_px, npix, params,
-                                                         chi2, sub);
-    return cudaGetLastError();
+    if (dtype == ME_F32)
+        return pb.fill ? chi2_t<float, true>(pb, obs, w, mu_px, npix, params, chi2, st, sub)
+                       : chi2_t<float, false>(pb, obs, w, mu_px, npix, params, chi2, st, sub);
+    return pb.fill ? chi2_t<double, true>(pb, obs, w, mu_px, npix, params, chi2, st, sub)
+                   : chi2_t<double, false>(pb, obs, w, mu_px, npix, params, chi2, st, sub);
 }
 
 }  // namespace genesis
