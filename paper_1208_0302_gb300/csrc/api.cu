@@ -196,6 +196,10 @@ int make_problem(const me_problem *pb, KProblem &k)
             }
         }
         k.line[l].zfacL = kZeeman * ln.lambda0_A * ln.lambda0_A;
+        k.line[l].lam0_c32 = (float)k.line[l].lam0_c;
+        k.line[l].dscale32 = (float)k.line[l].dscale;
+        k.line[l].zfac32 = (float)k.line[l].zfac;
+        k.line[l].zfacL32 = (float)k.line[l].zfacL;
         if (ln.pattern) {
             int rc = zeeman_pattern(ln.j_lower, ln.g_lower, ln.j_upper, ln.g_upper, k.line[l].ncomp,
                                     k.line[l].cshift, k.line[l].cstr);

@@ -58,31 +58,6 @@ __device__ __forceinline__ long long order64(double x)
     return b == (long long)0x8000000000000000ull ? 0 : b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
-__device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
-__device__ __forceinline__ double abs_of(double x) { return fabs(x); }
-__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
-
-// Correctly rounded a / b for a divisor whose correctly rounded reciprocal rb
-// is at hand (Markstein 1990): two quotient corrections by exact remainders,
-// five FP64 operations where the division takes 8 to 9.  rb = 0 marks a
-// divisor outside 2^+-200; those, and dividends outside 2^+-700 other than 0,
-// are divided outright (no remainder may underflow).
-__device__ __forceinline__ double div_known(double a, double b, double rb)
-{
-    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
-    const bool zero = (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) == 0u;
-    if (rb == 0.0 || !(zero || ea - 323u < 1400u)) return __ddiv_rn(a, b);
-    double q = __dmul_rn(a, rb);
-    q = __fma_rn(__fma_rn(-b, q, a), rb, q);
-    return __fma_rn(__fma_rn(-b, q, a), rb, q);
-}
-__device__ __forceinline__ double known_rcp(double b)
-{
-    const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
-    return eb - 823u < 400u ? __ddiv_rn(1.0, b) : 0.0;
-}
-
 constexpr int kChunk = 32;            // wavelengths staged at once
 constexpr int kPitch = kChunk + 1;    // tile row pitch: a column read touches 32 banks
 

@@ -38,4 +38,81 @@ __device__ __forceinline__ double rcp_newton(double d)
     return fma(r, fma(e, e, e), r);
 }
 
+// Correctly rounded a / b for a divisor whose correctly rounded reciprocal rb
+// is at hand (Markstein 1990): two quotient corrections by exact remainders,
+// five FP64 operations where the division takes 8 to 9.  rb = 0 marks a
+// divisor outside 2^+-200; those, and dividends outside 2^+-700 other than 0,
+// are divided outright (no remainder may underflow).
+__device__ __forceinline__ double div_known(double a, double b, double rb)
+{
+    const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu;
+    const bool zero = (((unsigned)__double2hiint(a) << 1) | (unsigned)__double2loint(a)) == 0u;
+    if (rb == 0.0 || !(zero || ea - 323u < 1400u)) return __ddiv_rn(a, b);
+    double q = __dmul_rn(a, rb);
+    q = __fma_rn(__fma_rn(-b, q, a), rb, q);
+    return __fma_rn(__fma_rn(-b, q, a), rb, q);
+}
+__device__ __forceinline__ double known_rcp(double b)
+{
+    const unsigned eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+    return eb - 823u < 400u ? __ddiv_rn(1.0, b) : 0.0;
+}
+
+__device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
+__device__ __forceinline__ double abs_of(double x) { return fabs(x); }
+__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
+__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
+
+// One warp: a pixel's squared weights into s_w2[4], the caller's or Section
+// 5.4's inverse-max weights in FP64 (the extrema in the cube's own type).
+template <class RO>
+__device__ __forceinline__ void weights64(const RO *o, int nl, const double *w_user, int pix, double *s_w2)
+{
+    const int lane = threadIdx.x & 31;
+    if (w_user) {
+        if (lane < 4) {
+            const double w = w_user[(size_t)pix * 4 + lane];
+            s_w2[lane] = w * w;
+        }
+        return;
+    }
+    RO imax = -INFINITY, nmin = -INFINITY, m[3] = {0, 0, 0};  // nmin = -min I
+    for (int j = lane; j < nl; j += 32) {
+        imax = max_of(imax, o[j]);
+        nmin = max_of(nmin, -o[j]);
+#pragma unroll
+        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], abs_of(o[(s + 1) * nl + j]));
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        imax = max_of(imax, __shfl_xor_sync(0xffffffffu, imax, off));
+        nmin = max_of(nmin, __shfl_xor_sync(0xffffffffu, nmin, off));
+#pragma unroll
+        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], __shfl_xor_sync(0xffffffffu, m[s], off));
+    }
+    if (lane < 4) {
+        const double top = (double)imax;
+        const double d = lane == 0 ? top + (double)nmin : (double)(lane == 1 ? m[0] : lane == 2 ? m[1] : m[2]);
+        const double fl = 1e-6 * fabs(top);
+        const double dd = d > fl ? d : fl;
+        const double w = dd > 0.0 ? 1.0 / dd : 0.0;
+        s_w2[lane] = w * w;
+    }
+}
+
+// The warp sums of four FP64 values at once: the butterfly's additions (lane
+// distances 16, 8, 4, 2, 1), but each lane keeps only the values it goes on
+// with, so that 6 additions do what 20 would.  Sum s lands on the eight lanes
+// with lane / 8 == s, the same bits that four butterflies give.
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3)
+{
+    const bool h16 = threadIdx.x & 16, h8 = threadIdx.x & 8;
+    const double x0 = (h16 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h16 ? v0 : v2, 16);
+    const double x1 = (h16 ? v3 : v1) + __shfl_xor_sync(0xffffffffu, h16 ? v1 : v3, 16);
+    double v = (h8 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, h8 ? x0 : x1, 8);
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+
 }  // namespace genesis

@@ -138,11 +138,11 @@ __device__ __forceinline__ R fitness_rows(const KProblem &pb, int nlines, int nl
 // individual's closed-form constants and w_I for the length of the call:
 // they are read once per pair instead of holding registers through the
 // profile evaluations.
-template <int NL, bool COUNT, bool PAT, bool FILL, bool STORE = false>
-__device__ __forceinline__ float fitness_pairs(const KProblem &pb, int nlines, int nl, const float *p,
-                                               float mu, const float *s_obs, const float *s_doff,
-                                               const float *he, const float *s_w2, float inv_nu,
-                                               WorkCount &wc, float4 *s_kc, float *res = nullptr)
+// The individual's geometry for the pair loop, its weights folded in and its
+// slots filled (k = its index, nt = the slots' stride).
+template <int NL, bool FILL>
+__device__ __forceinline__ Geo<float> pair_geometry(const KProblem &pb, int nlines, const float *p, float mu,
+                                                    const float *s_w2, float4 *s_kc, int k, int nt)
 {
     Geo<float> geo = make_geo<float, NL, FILL>(pb, nlines, p, mu);
     pair_thresholds(geo, nlines);
@@ -153,57 +153,106 @@ __device__ __forceinline__ float fitness_pairs(const KProblem &pb, int nlines, i
     geo.kU *= sw[2];
     geo.kQV *= sw[2];
     geo.kV *= sw[3];
+    s_kc[k] = make_float4(geo.kIs, geo.kIp, geo.kIp2, geo.kV2);
+    s_kc[nt + k] = make_float4(geo.muS1, geo.S0, geo.kQ, geo.kUV);
+    s_kc[2 * nt + k] = make_float4(geo.kU, geo.kQV, geo.kV, sw[0]);
+    return geo;
+}
+
+// The sum of pair q's eight squared weighted residuals.
+template <int NL, bool COUNT, bool PAT, bool FILL, bool STORE>
+__device__ __forceinline__ float pair_square(const KProblem &pb, int nlines, int nl, const Geo<float> &geo, int q,
+                                             const float *s_obs, const float *s_doff, const float *he,
+                                             EvalCount &cnt, const float4 *kc, int nt, float *res)
+{
+    const float4 d0 = *(const float4 *)(s_doff + 8 * q);
+    float2 doff2[ME_MAX_LINES];
+    doff2[0] = make_float2(d0.x, d0.y);
+    doff2[1] = make_float2(d0.z, d0.w);
+    if (NL == 0 || NL > 2) {
+        const float4 d1 = *(const float4 *)(s_doff + 8 * q + 4);
+        doff2[2] = make_float2(d1.x, d1.y);
+        doff2[3] = make_float2(d1.z, d1.w);
+    }
+    const bool y_real = 2 * q + 1 < nl;
+    float wIs;
+    const Stokes4x2 rr = resid_x2<NL, COUNT, PAT, FILL>(geo, doff2, s_obs + 8 * q, he, nlines, y_real, cnt, pb.line, kc, nt,
+                                                        wIs);
+    float2 rI = mul2(rr.I, f2(wIs)), rQ = rr.Q, rU = rr.U, rV = rr.V;
+    if (!y_real) rI.y = rQ.y = rU.y = rV.y = 0.f;  // padded partner
+    if (STORE && res) {
+        const int j = 2 * q;
+        res[j] = rI.x;
+        res[nl + j] = rQ.x;
+        res[2 * nl + j] = rU.x;
+        res[3 * nl + j] = rV.x;
+        if (y_real) {
+            res[j + 1] = rI.y;
+            res[nl + j + 1] = rQ.y;
+            res[2 * nl + j + 1] = rU.y;
+            res[3 * nl + j + 1] = rV.y;
+        }
+    }
+    float2 t2 = fma2(rQ, rQ, mul2(rI, rI));
+    t2 = fma2(rU, rU, t2);
+    t2 = fma2(rV, rV, t2);
+    return t2.x + t2.y;
+}
+
+// Kahan's update of the running total (comp holds the lost low part, negated).
+__device__ __forceinline__ void kahan_add(float &sum, float &comp, float v)
+{
+    const float y = v - comp;
+    const float t = sum + y;
+    comp = (t - sum) - y;
+    sum = t;
+}
+
+template <int NL, bool COUNT, bool PAT, bool FILL, bool STORE = false>
+__device__ __forceinline__ float fitness_pairs(const KProblem &pb, int nlines, int nl, const float *p,
+                                               float mu, const float *s_obs, const float *s_doff,
+                                               const float *he, const float *s_w2, float inv_nu,
+                                               WorkCount &wc, float4 *s_kc, float *res = nullptr)
+{
     const int kt = threadIdx.x, nt = blockDim.x;
-    s_kc[kt] = make_float4(geo.kIs, geo.kIp, geo.kIp2, geo.kV2);
-    s_kc[nt + kt] = make_float4(geo.muS1, geo.S0, geo.kQ, geo.kUV);
-    s_kc[2 * nt + kt] = make_float4(geo.kU, geo.kQV, geo.kV, sw[0]);
-    const float4 *kc = s_kc + kt;
+    const Geo<float> geo = pair_geometry<NL, FILL>(pb, nlines, p, mu, s_w2, s_kc, kt, nt);
     float sum = 0.f, comp = 0.f;
     const int npair = (nl + 1) >> 1;
     EvalCount cnt{0u, 0u, 0u, 0u};
-    for (int q = 0; q < npair; ++q) {
-        const float4 d0 = *(const float4 *)(s_doff + 8 * q);
-        float2 doff2[ME_MAX_LINES];
-        doff2[0] = make_float2(d0.x, d0.y);
-        doff2[1] = make_float2(d0.z, d0.w);
-        if (NL == 0 || NL > 2) {
-            const float4 d1 = *(const float4 *)(s_doff + 8 * q + 4);
-            doff2[2] = make_float2(d1.x, d1.y);
-            doff2[3] = make_float2(d1.z, d1.w);
-        }
-        const bool y_real = 2 * q + 1 < nl;
-        float wIs;
-        const Stokes4x2 rr = resid_x2<NL, COUNT, PAT, FILL>(geo, doff2, s_obs + 8 * q, he, nlines, y_real, cnt, pb.line, kc, nt,
-                                                            wIs);
-        float2 rI = mul2(rr.I, f2(wIs)), rQ = rr.Q, rU = rr.U, rV = rr.V;
-        if (!y_real) rI.y = rQ.y = rU.y = rV.y = 0.f;  // padded partner
-        if (STORE && res) {
-            const int j = 2 * q;
-            res[j] = rI.x;
-            res[nl + j] = rQ.x;
-            res[2 * nl + j] = rU.x;
-            res[3 * nl + j] = rV.x;
-            if (y_real) {
-                res[j + 1] = rI.y;
-                res[nl + j + 1] = rQ.y;
-                res[2 * nl + j + 1] = rU.y;
-                res[3 * nl + j + 1] = rV.y;
-            }
-        }
-        float2 t2 = fma2(rQ, rQ, mul2(rI, rI));
-        t2 = fma2(rU, rU, t2);
-        t2 = fma2(rV, rV, t2);
-        const float y = (t2.x + t2.y) - comp;  // Kahan: comp holds the lost low part, negated
-        const float t = sum + y;
-        comp = (t - sum) - y;
-        sum = t;
-    }
+    for (int q = 0; q < npair; ++q)
+        kahan_add(sum, comp, pair_square<NL, COUNT, PAT, FILL, STORE>(pb, nlines, nl, geo, q, s_obs, s_doff, he, cnt,
+                                                                      s_kc + kt, nt, res));
     if (COUNT) {
         wc.interior += cnt.interior;
         wc.mid += cnt.mid;
         wc.even2 += cnt.even2;
         wc.far += cnt.far;
     }
+    return (sum - comp) * inv_nu;
+}
+
+// A split block's share of one individual's pairs: segment seg of nseg takes
+// pairs seg, seg + nseg, ... and leaves each pair's sum in s_part[q npop + k];
+// after a barrier sum_parts adds them in the order of fitness_pairs.
+template <int NL, bool PAT, bool FILL>
+__device__ __forceinline__ void fitness_share(const KProblem &pb, int nlines, int nl, const float *p, float mu,
+                                              const float *s_obs, const float *s_doff, const float *he,
+                                              const float *s_w2, float4 *s_kc, float *s_part, int k, int npop,
+                                              int seg, int nseg)
+{
+    const Geo<float> geo = pair_geometry<NL, FILL>(pb, nlines, p, mu, s_w2, s_kc, k, npop);
+    const int npair = (nl + 1) >> 1;
+    EvalCount cnt{0u, 0u, 0u, 0u};
+    for (int q = seg; q < npair; q += nseg)
+        s_part[q * npop + k] = pair_square<NL, false, PAT, FILL, false>(pb, nlines, nl, geo, q, s_obs, s_doff, he, cnt,
+                                                                        s_kc + k, npop, nullptr);
+}
+__device__ __forceinline__ float sum_parts(const float *s_part, int nl, int npop, int k, float inv_nu)
+{
+    float sum = 0.f, comp = 0.f;
+    const int npair = (nl + 1) >> 1;
+#pragma unroll 8
+    for (int q = 0; q < npair; ++q) kahan_add(sum, comp, s_part[q * npop + k]);
     return (sum - comp) * inv_nu;
 }
 
@@ -220,21 +269,23 @@ __device__ __forceinline__ R fitness(const KProblem &pb, int nlines, int nl, con
                                                             inv_nu, wc, res);
 }
 
-// argmin over the block's fitness, ties to the lowest index.  Every thread
-// gets the result.  Uses one __syncthreads().
+// argmin over the block's npop fitness values, ties to the lowest index.
+// Every thread gets the result.  Uses one __syncthreads().
 template <class R>
-__device__ __forceinline__ int block_argmin(const R *s_fit, R *s_wmin, int *s_widx)
+__device__ __forceinline__ int block_argmin(const R *s_fit, int npop, R *s_wmin, int *s_widx)
 {
-    const int k = threadIdx.x, lane = k & 31, warp = k >> 5, nw = blockDim.x >> 5;
-    R v = s_fit[k];
-    int idx = k;
+    const int k = threadIdx.x, lane = k & 31, warp = k >> 5, nw = npop >> 5;
+    if (k < npop) {
+        R v = s_fit[k];
+        int idx = k;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const R ov = __shfl_down_sync(0xffffffffu, v, off);
-        const int oi = __shfl_down_sync(0xffffffffu, idx, off);
-        if (ov < v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+        for (int off = 16; off > 0; off >>= 1) {
+            const R ov = __shfl_down_sync(0xffffffffu, v, off);
+            const int oi = __shfl_down_sync(0xffffffffu, idx, off);
+            if (ov < v || (ov == v && oi < idx)) { v = ov; idx = oi; }
+        }
+        if (lane == 0) { s_wmin[warp] = v; s_widx[warp] = idx; }
     }
-    if (lane == 0) { s_wmin[warp] = v; s_widx[warp] = idx; }
     __syncthreads();
     R bv = s_wmin[0];
     int bi = s_widx[0];
@@ -343,11 +394,11 @@ __device__ __forceinline__ void breed_one(const KGa &ga, uint64_t pid, int t, in
 
 struct GaSmem {
     // byte offsets into dynamic shared memory
-    int obs, doff, fit, wmin, widx, w2, he, dom, genes, kc, total;
+    int obs, doff, fit, wmin, widx, w2, he, dom, genes, kc, part, total;
 };
 
 template <class R>
-__host__ __device__ __forceinline__ GaSmem ga_smem_layout(int nl, int nlines, int npop, int npar)
+__host__ __device__ __forceinline__ GaSmem ga_smem_layout(int nl, int nlines, int npop, int npar, bool split = false)
 {
     GaSmem L;
     int o = 0;
@@ -368,6 +419,7 @@ __host__ __device__ __forceinline__ GaSmem ga_smem_layout(int nl, int nlines, in
     L.dom = take((int)sizeof(DecodeDomain), 16);  // the pixel's decode domain
     L.genes = take(2 * npop * npar * 2, 16);
     L.kc = take(sizeof(R) == 4 ? 3 * npop * 16 : 0, 16);  // FP32: 3 float4 of closed-form constants per thread
+    L.part = take(split ? (nl + 1) / 2 * npop * 4 : 0, 16);  // a split block's pair sums
     L.total = (o + 15) / 16 * 16;
     return L;
 }
@@ -508,7 +560,15 @@ __device__ __forceinline__ void weight_obs_rows(R *s_obs, int nl, int k, const R
                              : (sizeof(R) == 4 ? ((NL) > 0 && !(PAT) ? GENESIS_GA_NREG32 : 80) : 255))
 #endif
 
-template <class R, int NL, int MAXT, bool COUNT, bool PAT, int M>
+// SPLIT (FP32): blockDim.x / npop threads per individual share its wavelength
+// pairs.  With fewer pixels than fill the chip at a block of npop threads
+// each, an SM holds only a few warps and the fitness loop is a chain of
+// dependent operations; the shares run side by side.  A pair is evaluated by
+// the same lanes of a warp as without the split (so its votes, and with them
+// its bits, are the same), and the pairs' sums are added in the same order by
+// one thread, so the result does not depend on the split.  64 pixels,
+// population 64, 100 generations: 4.25 -> 1.68 ms.
+template <class R, int NL, int MAXT, bool COUNT, bool PAT, int M, bool SPLIT>
 __global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT)
 k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
             const R *__restrict__ obs, const double *__restrict__ w_user,
@@ -523,8 +583,10 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     const int nl = pb.n_lambda;
     const int nlines = NL > 0 ? NL : pb.n_lines;
     const int npop = ga.npop;
-    const int k = threadIdx.x;
-    const GaSmem L = ga_smem_layout<R>(nl, nlines, npop, M);
+    const int tid = threadIdx.x;
+    const int seg = SPLIT ? tid / npop : 0, nseg = SPLIT ? blockDim.x / npop : 1;
+    const int k = SPLIT ? tid - seg * npop : tid;  // individual
+    const GaSmem L = ga_smem_layout<R>(nl, nlines, npop, M, SPLIT);
     R *s_obs = (R *)(smem + L.obs);
     R *s_doff = (R *)(smem + L.doff);
     R *s_fit = (R *)(smem + L.fit);
@@ -535,32 +597,33 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     DecodeDomain &D = *(DecodeDomain *)(smem + L.dom);
     uint16_t *s_genes = (uint16_t *)(smem + L.genes);
     float4 *s_kc = (float4 *)(smem + L.kc);
+    float *s_part = (float *)(smem + L.part);
 
     // per-launch constants
     const R inv_nu = R(1) / R(4 * nl - M);
-    stage_offsets_ga<R>(pb, nlines, nl, k, s_doff, s_he);
+    stage_offsets_ga<R>(pb, nlines, nl, tid, s_doff, s_he);
 
     const int nrun = sub.count ? min(*sub.count, npix) : npix;
     for (int blk = blockIdx.x; blk < nrun; blk += gridDim.x) {
         const int pix = sub.index ? sub.index[blk] : blk;
         if (pix < 0 || pix >= npix) continue;  // a bad index skips the block, uniformly
-        if (k < M) {  // the pixel's decode domain of parameter k
-            double a = sd.bounds_px ? sd.bounds_px[(size_t)pix * 2 * M + k] : ga.lo[k];
-            double b = sd.bounds_px ? sd.bounds_px[(size_t)pix * 2 * M + M + k] : ga.hi[k];
-            if (k == 1 && sd.polarity) polarity_bounds(sd.polarity[pix], a, b, a, b);
-            D.lo[k] = a;
-            D.hi[k] = b;
-            D.lo32[k] = (float)a;
-            D.sc32[k] = (float)((b - a) / 65535.0);
+        if (tid < M) {  // the pixel's decode domain of parameter tid
+            double a = sd.bounds_px ? sd.bounds_px[(size_t)pix * 2 * M + tid] : ga.lo[tid];
+            double b = sd.bounds_px ? sd.bounds_px[(size_t)pix * 2 * M + M + tid] : ga.hi[tid];
+            if (tid == 1 && sd.polarity) polarity_bounds(sd.polarity[pix], a, b, a, b);
+            D.lo[tid] = a;
+            D.hi[tid] = b;
+            D.lo32[tid] = (float)a;
+            D.sc32[tid] = (float)((b - a) / 65535.0);
         }
         // a1: stage the pixel's Stokes profiles
-        stage_obs<R>(obs + (size_t)pix * 4 * nl, nl, k, s_obs);
+        stage_obs<R>(obs + (size_t)pix * 4 * nl, nl, tid, s_obs);
         __syncthreads();
         // a2: weights
-        stage_weights<R>(ga.weight_mode, w_user, pix, s_obs, nl, k, s_w2);
+        stage_weights<R>(ga.weight_mode, w_user, pix, s_obs, nl, tid, s_w2);
         __syncthreads();
         if (sizeof(R) == 4) {
-            weight_obs_rows<R>(s_obs, nl, k, s_w2);
+            weight_obs_rows<R>(s_obs, nl, tid, s_w2);
             __syncthreads();
         }
         R he[ME_MAX_LINES];
@@ -568,6 +631,18 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
         for (int l = 0; l < ME_MAX_LINES; ++l) he[l] = s_he[l];
         const R mu = mu_px ? R(mu_px[pix]) : R(pb.mu);
         const uint64_t pid = ga.pixel_id0 + (uint64_t)pix;
+        // p's fitness into s_fit[slot], for the individuals that are on (the
+        // same ones in every segment); with SPLIT one barrier inside
+        auto evaluate = [&](const R *p, bool on, int slot) {
+            if constexpr (SPLIT) {
+                if (on) fitness_share<NL, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, s_kc, s_part, k, npop, seg, nseg);
+                __syncthreads();
+                if (on && seg == 0) s_fit[slot] = clean_fit(sum_parts(s_part, nl, npop, k, inv_nu));
+            } else if (on) {
+                s_fit[slot] = clean_fit(fitness<R, NL, COUNT, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu, wc, s_kc));
+                if (COUNT) ++nfit;
+            }
+        };
 
         // a3 + a4: Sobol points 1..npop, the last nseed taking the seeds'
         // (B, psi, chi) genes, decode, evaluate
@@ -585,62 +660,70 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
 #pragma unroll
         for (int d = 0; d < M; ++d) p[d] = GaDecode<R>::get(D, d, g[d]);
         int cur = 0;
+        if (seg == 0) {
 #pragma unroll
-        for (int d = 0; d < M; ++d) s_genes[k * M + d] = g[d];
-        s_fit[k] = clean_fit(fitness<R, NL, COUNT, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu, wc, s_kc));
-        if (COUNT) ++nfit;
+            for (int d = 0; d < M; ++d) s_genes[k * M + d] = g[d];
+        }
+        evaluate(p, true, k);
         uint64_t sobol_next = (uint64_t)npop + 1;
 
         for (int t = 1; t <= ga.ngen; ++t) {
             __syncthreads();  // fitness and genes of generation t-1 complete
-            const int elite = block_argmin<R>(s_fit, s_wmin, s_widx);  // a9
+            const int elite = block_argmin<R>(s_fit, npop, s_wmin, s_widx);  // a9
             const uint16_t *s_cur = s_genes + cur * npop * M;
             uint16_t *s_nxt = s_genes + (cur ^ 1) * npop * M;
-            breed_one<R, M>(ga, pid, t, k, npop, s_fit, s_cur, elite, s_nxt + k * M, g);  // a10-a12
+            if (seg == 0) {
+                breed_one<R, M>(ga, pid, t, k, npop, s_fit, s_cur, elite, s_nxt + k * M, g);  // a10-a12
+                if (SPLIT) {
+#pragma unroll
+                    for (int d = 0; d < M; ++d) s_nxt[k * M + d] = g[d];
+                }
+            }
             __syncthreads();  // every tournament has read s_fit
 #pragma unroll
             for (int d = 0; d < M; ++d) {
-                s_nxt[k * M + d] = g[d];
+                if (SPLIT) g[d] = s_nxt[k * M + d];
+                else s_nxt[k * M + d] = g[d];
                 p[d] = GaDecode<R>::get(D, d, g[d]);
             }
             cur ^= 1;
-            s_fit[k] = clean_fit(fitness<R, NL, COUNT, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu, wc, s_kc));
-            if (COUNT) ++nfit;
+            evaluate(p, true, k);
             // a13: worst-half Sobol restart.  The individual of rank npop/2 + i
             // takes Sobol point sobol_next + i; thread i evaluates it, so the
             // new half fills whole warps (the idle half of the gene double
             // buffer carries the individuals' indices).
             if (ga.nsamp > 0 && t % ga.nsamp == 0 && t < ga.ngen) {
                 __syncthreads();
-                const int rank = stable_rank<R>(s_fit, npop, k);
                 int *s_ridx = (int *)(s_genes + (cur ^ 1) * npop * M);
-                if (rank >= npop / 2) s_ridx[rank - npop / 2] = k;
+                if (seg == 0) {
+                    const int rank = stable_rank<R>(s_fit, npop, k);
+                    if (rank >= npop / 2) s_ridx[rank - npop / 2] = k;
+                }
                 __syncthreads();
-                if (k < npop / 2) {
-                    const int kr = s_ridx[k];
+                const bool on = k < npop / 2;
+                int kr = k;
+                if (on) {
+                    kr = s_ridx[k];
                     const uint64_t n = sobol_next + (uint64_t)k;
                     uint16_t *s_c = s_genes + cur * npop * M;
 #pragma unroll
                     for (int d = 0; d < M; ++d) {
                         g[d] = (uint16_t)(sobol_point(n, d) >> 16);
-                        s_c[kr * M + d] = g[d];
+                        if (seg == 0) s_c[kr * M + d] = g[d];
                         p[d] = GaDecode<R>::get(D, d, g[d]);
                     }
-                    s_fit[kr] = clean_fit(
-                        fitness<R, NL, COUNT, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu, wc, s_kc));
-                    if (COUNT) ++nfit;
                 }
+                evaluate(p, on, kr);
                 sobol_next += (uint64_t)(npop / 2);
             }
         }
         __syncthreads();
-        const int b = block_argmin<R>(s_fit, s_wmin, s_widx);
+        const int b = block_argmin<R>(s_fit, npop, s_wmin, s_widx);
         // a14: decoded best individual (its FP64 chi2 is a separate pass)
-        if (k < M) {
-            const uint16_t gb = s_genes[cur * npop * M + b * M + k];
-            best[(size_t)pix * M + k] =
-                decode64(gb, D.lo[k], D.hi[k]);
-            if (best_genes) best_genes[(size_t)pix * M + k] = gb;
+        if (tid < M) {
+            const uint16_t gb = s_genes[cur * npop * M + b * M + tid];
+            best[(size_t)pix * M + tid] = decode64(gb, D.lo[tid], D.hi[tid]);
+            if (best_genes) best_genes[(size_t)pix * M + tid] = gb;
         }
         __syncthreads();  // shared memory is reused by the next pixel
     }
@@ -661,6 +744,16 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     }
 }
 
+// Threads per individual for npix pixels: as many as keep an SM's share of
+// the pixels within the warps its registers hold (28 at 72 registers, 24 at
+// 80); 1 = no split.
+inline int ga_segments(int npix, int npop, int nl, int regs)
+{
+    const int warps = regs <= 72 ? 28 : 24, per_sm = (npix + 151) / 152;
+    const int s = warps / (per_sm * (npop / 32)), npair = (nl + 1) / 2;
+    return s < npair ? s : npair;
+}
+
 template <class R, int NL, int MAXT, bool COUNT = false, bool PAT = false, int M = ME_NPAR>
 cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, const double *w,
                             const double *mu_px, int npix, double *best, uint16_t *best_genes,
@@ -668,8 +761,20 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
                             KSub sub = {})
 {
     const int nlines = NL > 0 ? NL : pb.n_lines;
+    if constexpr (sizeof(R) == 4 && MAXT <= 256 && !COUNT) {
+        const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, NL > 0 && !PAT ? GENESIS_GA_NREG32 : 80);
+        const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M, true);
+        if (nseg > 1 && L.total <= 200 * 1024) {
+            auto kern = k_ga_evolve<R, NL, MAXT, false, PAT, M, true>;
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+            if (e != cudaSuccess) return e;
+            kern<<<npix, nseg * ga.npop, L.total, st>>>(pb, ga, (const R *)obs, w, mu_px, npix, best, best_genes,
+                                                        counts, sd, sub);
+            return cudaGetLastError();
+        }
+    }
     const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M);
-    auto kern = k_ga_evolve<R, NL, MAXT, COUNT, PAT, M>;
+    auto kern = k_ga_evolve<R, NL, MAXT, COUNT, PAT, M, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
     if (e != cudaSuccess) return e;
     kern<<<npix, ga.npop, L.total, st>>>(pb, ga, (const R *)obs, w, mu_px, npix, best, best_genes, counts,

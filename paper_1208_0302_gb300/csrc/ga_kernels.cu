@@ -39,7 +39,7 @@ __global__ void k_ga_breed(const __grid_constant__ KGa ga, const uint16_t *__res
 #pragma unroll
     for (int d = 0; d < M; ++d) s_cur[k * M + d] = genes[(base + k) * M + d];
     __syncthreads();
-    const int elite = block_argmin<double>(s_fit, s_wmin, s_widx);
+    const int elite = block_argmin<double>(s_fit, npop, s_wmin, s_widx);
     uint16_t g[M];
     breed_one<double, M>(ga, ga.pixel_id0 + (uint64_t)prob, gen, k, npop, s_fit, s_cur, elite,
                       s_new + k * M, g);

@@ -30,6 +30,7 @@ struct KLine {
     double cstr[3][ME_MAX_COMP];    // component strengths (sum 1 per group)
     float cshift32[3][ME_MAX_COMP];
     float cstr32[3][ME_MAX_COMP];
+    float lam0_c32, dscale32, zfac32, zfacL32;  // the FP64 constants rounded (a conversion takes the FP64 pipe)
     float2 qs2;        // FP32 pair path: half_eta / sqrt(pi) in both lanes
     float2 wq2[17];    // FP32 pair path: Weideman coefficients 2 a_n times half_eta, in both lanes
 };
@@ -40,6 +41,11 @@ template <> __device__ __forceinline__ double comp_shift<double>(const KLine &ln
 template <class R> __device__ __forceinline__ R comp_str(const KLine &ln, int g, int i);
 template <> __device__ __forceinline__ float comp_str<float>(const KLine &ln, int g, int i) { return ln.cstr32[g][i]; }
 template <> __device__ __forceinline__ double comp_str<double>(const KLine &ln, int g, int i) { return ln.cstr[g][i]; }
+
+template <class R> __device__ __forceinline__ R line_lam0_c(const KLine &ln) { return sizeof(R) == 4 ? R(ln.lam0_c32) : R(ln.lam0_c); }
+template <class R> __device__ __forceinline__ R line_dscale(const KLine &ln) { return sizeof(R) == 4 ? R(ln.dscale32) : R(ln.dscale); }
+template <class R> __device__ __forceinline__ R line_zfac(const KLine &ln) { return sizeof(R) == 4 ? R(ln.zfac32) : R(ln.zfac); }
+template <class R> __device__ __forceinline__ R line_zfacL(const KLine &ln) { return sizeof(R) == 4 ? R(ln.zfacL32) : R(ln.zfacL); }
 
 // Everything a synthesis needs, passed by value in the kernel parameters
 // (about 6.4 KB, within the 32 KB parameter space of sm_70+).
@@ -308,11 +314,11 @@ __device__ __forceinline__ Geo<R> make_geo(const KProblem &pb, int nlines, const
     for (int l = 0; l < (NL > 0 ? NL : ME_MAX_LINES); ++l) {
         if (l < nl) {
             const KLine &ln = pb.line[l];
-            g.shift[l] = R(ln.lam0_c) * p[3];
-            g.invD[l] = R(1) / (p[4] * R(ln.dscale));
-            g.vB[l] = R(ln.zfac) * p[0] * g.invD[l];
+            g.shift[l] = line_lam0_c<R>(ln) * p[3];
+            g.invD[l] = R(1) / (p[4] * line_dscale<R>(ln));
+            g.vB[l] = line_zfac<R>(ln) * p[0] * g.invD[l];
             g.cp[l] = -g.shift[l] * g.invD[l];
-            g.vL[l] = R(ln.zfacL) * p[0] * g.invD[l];
+            g.vL[l] = line_zfacL<R>(ln) * p[0] * g.invD[l];
         }
     }
     return g;

@@ -50,9 +50,9 @@ __device__ __forceinline__ GeoJ<R> make_geoj(const KProblem &pb, int nlines, con
 #pragma unroll
     for (int l = 0; l < (NL > 0 ? NL : ME_MAX_LINES); ++l) {
         if (l < nl) {
-            G.kv[l] = R(pb.line[l].lam0_c) * G.g.invD[l];
-            G.kB[l] = R(pb.line[l].zfac) * G.g.invD[l];
-            G.kL[l] = R(pb.line[l].zfacL) * G.g.invD[l];
+            G.kv[l] = line_lam0_c<R>(pb.line[l]) * G.g.invD[l];
+            G.kB[l] = line_zfac<R>(pb.line[l]) * G.g.invD[l];
+            G.kL[l] = line_zfacL<R>(pb.line[l]) * G.g.invD[l];
         }
     }
     return G;

@@ -199,48 +199,6 @@ k_synth64(const __grid_constant__ KProblem pb, const double *__restrict__ params
     }
 }
 
-__device__ __forceinline__ float abs_of(float x) { return fabsf(x); }
-__device__ __forceinline__ double abs_of(double x) { return fabs(x); }
-__device__ __forceinline__ float max_of(float a, float b) { return fmaxf(a, b); }
-__device__ __forceinline__ double max_of(double a, double b) { return fmax(a, b); }
-
-// One warp: the pixel's squared weights, the caller's or Section 5.4's
-// inverse-max weights in FP64 (the extrema in the cube's own type).
-template <class RO>
-__device__ __forceinline__ void weights64(const RO *o, int nl, const double *w_user, int pix, double *s_w2)
-{
-    const int lane = threadIdx.x & 31;
-    if (w_user) {
-        if (lane < 4) {
-            const double w = w_user[(size_t)pix * 4 + lane];
-            s_w2[lane] = w * w;
-        }
-        return;
-    }
-    RO imax = -INFINITY, nmin = -INFINITY, m[3] = {0, 0, 0};  // nmin = -min I
-    for (int j = lane; j < nl; j += 32) {
-        imax = max_of(imax, o[j]);
-        nmin = max_of(nmin, -o[j]);
-#pragma unroll
-        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], abs_of(o[(s + 1) * nl + j]));
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        imax = max_of(imax, __shfl_xor_sync(0xffffffffu, imax, off));
-        nmin = max_of(nmin, __shfl_xor_sync(0xffffffffu, nmin, off));
-#pragma unroll
-        for (int s = 0; s < 3; ++s) m[s] = max_of(m[s], __shfl_xor_sync(0xffffffffu, m[s], off));
-    }
-    if (lane < 4) {
-        const double top = (double)imax;
-        const double d = lane == 0 ? top + (double)nmin : (double)(lane == 1 ? m[0] : lane == 2 ? m[1] : m[2]);
-        const double fl = 1e-6 * fabs(top);
-        const double dd = d > fl ? d : fl;
-        const double w = dd > 0.0 ? 1.0 / dd : 0.0;
-        s_w2[lane] = w * w;
-    }
-}
-
 // FP64 chi-square (Eq. chisq) of given parameters, one block per pixel,
 // threads over wavelengths, on the profiles of profiles64.cuh.  Bound by the
 // FP64 pipe: 65 536 two-line pixels took 13.5 ms with Weideman's series and
@@ -283,14 +241,7 @@ k_chi2_f64(const __grid_constant__ KProblem pb, const RO *__restrict__ obs,
             ss[3] += r3 * r3;
         }
     }
-    // the four warp sums at once, halving the values a lane holds with the
-    // lanes it is added from: 6 FP64 additions instead of 20
-    const bool h16 = lane & 16, h8 = lane & 8;
-    const double x0 = (h16 ? ss[2] : ss[0]) + __shfl_xor_sync(0xffffffffu, h16 ? ss[0] : ss[2], 16);
-    const double x1 = (h16 ? ss[3] : ss[1]) + __shfl_xor_sync(0xffffffffu, h16 ? ss[1] : ss[3], 16);
-    double v = (h8 ? x1 : x0) + __shfl_xor_sync(0xffffffffu, h8 ? x0 : x1, 8);
-#pragma unroll
-    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    const double v = warp_sum4(ss[0], ss[1], ss[2], ss[3]);
     if ((lane & 7) == 0) s_red[warp][lane >> 3] = v;
     __syncthreads();
     if (warp == 0) {
