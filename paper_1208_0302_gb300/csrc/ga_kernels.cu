@@ -34,6 +34,8 @@ __global__ void k_ga_breed(const __grid_constant__ KGa ga, const uint16_t *__res
     int *s_widx = (int *)(s_wmin + 32);
     uint16_t *s_cur = (uint16_t *)(s_widx + 32);
     uint16_t *s_new = s_cur + npop * M;
+    __shared__ uint64_t s_tmut[136];
+    for (int i = k; i < 136; i += npop) s_tmut[i] = ga.t_mut[i];
     const size_t base = (size_t)prob * npop;
     s_fit[k] = clean_fit(fit[base + k]);
 #pragma unroll
@@ -42,7 +44,7 @@ __global__ void k_ga_breed(const __grid_constant__ KGa ga, const uint16_t *__res
     const int elite = block_argmin<double>(s_fit, npop, s_wmin, s_widx);
     uint16_t g[M];
     breed_one<double, M>(ga, ga.pixel_id0 + (uint64_t)prob, gen, k, npop, s_fit, s_cur, elite,
-                      s_new + k * M, g);
+                      s_tmut, s_new + k * M, g);
 #pragma unroll
     for (int d = 0; d < M; ++d) child[(base + k) * M + d] = g[d];
     if (k == 0 && elite_out) elite_out[prob] = elite;
