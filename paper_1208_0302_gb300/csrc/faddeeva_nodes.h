@@ -14,9 +14,9 @@
 
 namespace genesis {
 
-constexpr int kNodeGrid = 65;             // nodes per axis
-constexpr double kNodeStep = 0.15625;     // 10 / 64, exact
-constexpr int kNodeCoef = 14;             // coefficients kept per node
+constexpr int kNodeGrid = 129;            // nodes per axis
+constexpr double kNodeStep = 0.078125;    // 10 / 128, exact
+constexpr int kNodeCoef = 11;             // coefficients kept per node
 
 namespace nodes {
 
@@ -57,7 +57,7 @@ inline DD div(DD a, DD b)
 struct CDD {
     DD re, im;
 };
-constexpr int kTerms = 30;  // terms of a step: the first omitted is below 1e-32
+constexpr int kTerms = 24;  // terms of a step: the first omitted is below 1e-34
 
 // c_0 .. c_{kTerms-1} at z = x + i y from w = w(z).
 inline void taylor(double x, double y, CDD w, CDD c[kTerms])
@@ -78,7 +78,8 @@ inline void taylor(double x, double y, CDD w, CDD c[kTerms])
 
 }  // namespace nodes
 
-// Row (iy, ix) holds (re, im) of c_0 .. c_13 at z = ix step + i iy step.
+// Row (iy, ix) holds (re, im) of c_0 .. c_10 at z = ix step + i iy step.  At
+// most half a step away on each axis the first omitted term is below 5e-17.
 inline std::vector<double> faddeeva_nodes()
 {
     using namespace nodes;

@@ -20,7 +20,7 @@ namespace {
 // evaluate inside a divergent branch, as the GA's restarts do, so the pair
 // path's votes run over exactly those lanes.
 template <class R, int NL, int MAXT, bool PAT, int M>
-__global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT)
+__global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, false)
 k_ga_fitness(const __grid_constant__ KProblem pb, int weight_mode, const R *__restrict__ obs,
              const double *__restrict__ w_user, const double *__restrict__ mu_px, int nactive,
              const double *__restrict__ params, double *__restrict__ fit, R *__restrict__ res)
@@ -55,9 +55,20 @@ k_ga_fitness(const __grid_constant__ KProblem pb, int weight_mode, const R *__re
         R p[M];
 #pragma unroll
         for (int d = 0; d < M; ++d) p[d] = R(params[ind * M + d]);
-        WorkCount wc{};
-        const R f = fitness<R, NL, false, PAT, FILL, true>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu,
-                                                           wc, s_kc, res ? res + ind * 4 * nl : nullptr);
+        R *out = res ? res + ind * 4 * nl : nullptr;
+        R f;
+        if constexpr (sizeof(R) == 8 && MAXT <= 256) {
+            const Fit64Shared F = {(double *)(smem + L.f64), (double *)(smem + L.f64) + kF64Rows * npop, npop};
+            const Fit64Model m = fit64_model<FILL>(pb, p, mu);
+            fit64_coefficients(F, k, m.g.a, 0, 1);
+            for (int r = 0; r < kShares; ++r)
+                F.part[r * npop + k] = fit64_share<FILL, true>(pb, nl, m, F.coef + k, npop, s_obs, s_doff, s_w2, r, out);
+            f = fit64_total(F.part, npop, k, inv_nu);
+        } else {
+            WorkCount wc{};
+            f = fitness<R, NL, false, PAT, FILL, true>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, inv_nu, wc, s_kc,
+                                                       out);
+        }
         fit[ind] = double(f);
     }
 }

@@ -14,6 +14,7 @@
 
 #include <type_traits>
 
+#include "fitness64.cuh"
 #include "kernels.h"
 #include "me_pair.cuh"
 #include "rng_device.cuh"
@@ -396,7 +397,7 @@ __device__ __forceinline__ void breed_one(const KGa &ga, uint64_t pid, int t, in
 
 struct GaSmem {
     // byte offsets into dynamic shared memory
-    int obs, doff, fit, wmin, widx, w2, he, dom, tmut, genes, kc, part, total;
+    int obs, doff, fit, wmin, widx, w2, he, dom, tmut, genes, kc, part, f64, total;
 };
 
 template <class R>
@@ -422,7 +423,8 @@ __host__ __device__ __forceinline__ GaSmem ga_smem_layout(int nl, int nlines, in
     L.tmut = take(136 * 8, 16);                   // mutation thresholds
     L.genes = take(2 * npop * npar * 2, 16);
     L.kc = take(sizeof(R) == 4 ? 3 * npop * 16 : 0, 16);  // FP32: 3 float4 of closed-form constants per thread
-    L.part = take(split ? (nl + 1) / 2 * npop * 4 : 0, 16);  // a split block's pair sums
+    L.part = take(sizeof(R) == 4 && split ? (nl + 1) / 2 * npop * 4 : 0, 16);  // FP32: a split block's pair sums
+    L.f64 = take(sizeof(R) == 8 && npop <= 256 ? fit64_doubles(npop) * 8 : 0, 16);  // FP64: see Fit64Shared
     L.total = (o + 15) / 16 * 16;
     return L;
 }
@@ -549,22 +551,23 @@ __device__ __forceinline__ void weight_obs_rows(R *s_obs, int nl, int k, const R
 // is still 0.5 % faster than six blocks at 80 registers).  The other FP32
 // ones for npop <= 256 (any line count, full patterns) keep 80, where they
 // spill less.  1024-thread instantiations: 64, so that a whole block fits.
-// FP64 ones are bound by the FP64 units and may use up to 255.
+// FP64 ones are bound by the FP64 units and may use up to 255, or 128 where
+// a split block of up to 512 threads has to fit.
 #ifndef GENESIS_GA_NREG32
 #define GENESIS_GA_NREG32 72
 #endif
 // Build option: GENESIS_GA_MAXNREG=N caps every instantiation at N registers
 // per thread instead (for tuning the cap).
 #ifdef GENESIS_GA_MAXNREG
-#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT) __maxnreg__(GENESIS_GA_MAXNREG)
+#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT) __maxnreg__(GENESIS_GA_MAXNREG)
 #else
-#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT)                                                         \
+#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT)                                                  \
     __maxnreg__((MAXT) > 256 ? 65536 / (MAXT)                                                     \
-                             : (sizeof(R) == 4 ? ((NL) > 0 && !(PAT) ? GENESIS_GA_NREG32 : 80) : 255))
+                             : (sizeof(R) == 4 ? ((NL) > 0 && !(PAT) ? GENESIS_GA_NREG32 : 80) : (SPLIT) ? 128 : 255))
 #endif
 
-// SPLIT (FP32): blockDim.x / npop threads per individual share its wavelength
-// pairs.  With fewer pixels than fill the chip at a block of npop threads
+// SPLIT: blockDim.x / npop threads per individual share its wavelengths (FP32:
+// pairs; FP64: the shares of fitness64.cuh).  With fewer pixels than fill the chip at a block of npop threads
 // each, an SM holds only a few warps and the fitness loop is a chain of
 // dependent operations; the shares run side by side.  A pair is evaluated by
 // the same lanes of a warp as without the split (so its votes, and with them
@@ -572,7 +575,7 @@ __device__ __forceinline__ void weight_obs_rows(R *s_obs, int nl, int k, const R
 // one thread, so the result does not depend on the split.  64 pixels,
 // population 64, 100 generations: 4.25 -> 1.68 ms.
 template <class R, int NL, int MAXT, bool COUNT, bool PAT, int M, bool SPLIT>
-__global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT)
+__global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT)
 k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
             const R *__restrict__ obs, const double *__restrict__ w_user,
             const double *__restrict__ mu_px, int npix, double *__restrict__ best,
@@ -602,6 +605,8 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     float4 *s_kc = (float4 *)(smem + L.kc);
     float *s_part = (float *)(smem + L.part);
     uint64_t *s_tmut = (uint64_t *)(smem + L.tmut);
+    constexpr bool kFit64 = sizeof(R) == 8 && MAXT <= 256;
+    const Fit64Shared F = {(double *)(smem + L.f64), (double *)(smem + L.f64) + kF64Rows * npop, npop};
 
     // per-launch constants
     const R inv_nu = R(1) / R(4 * nl - M);
@@ -637,9 +642,21 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
         const R mu = mu_px ? R(mu_px[pix]) : R(pb.mu);
         const uint64_t pid = ga.pixel_id0 + (uint64_t)pix;
         // p's fitness into s_fit[slot], for the individuals that are on (the
-        // same ones in every segment); with SPLIT one barrier inside
+        // same ones in every segment); with SPLIT barriers inside
         auto evaluate = [&](const R *p, bool on, int slot) {
-            if constexpr (SPLIT) {
+            if constexpr (kFit64) {
+                Fit64Model m;
+                if (on) {
+                    m = fit64_model<FILL>(pb, p, mu);
+                    fit64_coefficients(F, k, m.g.a, seg, nseg);
+                }
+                if (SPLIT) __syncthreads();
+                if (on)
+                    for (int r = seg; r < kShares; r += nseg)
+                        F.part[r * npop + k] = fit64_share<FILL, false>(pb, nl, m, F.coef + k, npop, s_obs, s_doff, s_w2, r, nullptr);
+                if (SPLIT) __syncthreads();
+                if (on && seg == 0) s_fit[slot] = clean_fit(fit64_total(F.part, npop, k, inv_nu));
+            } else if constexpr (SPLIT) {
                 if (on) fitness_share<NL, PAT, FILL>(pb, nlines, nl, p, mu, s_obs, s_doff, he, s_w2, s_kc, s_part, k, npop, seg, nseg);
                 __syncthreads();
                 if (on && seg == 0) s_fit[slot] = clean_fit(sum_parts(s_part, nl, npop, k, inv_nu));
@@ -750,12 +767,14 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
 }
 
 // Threads per individual for npix pixels: as many as keep an SM's share of
-// the pixels within the warps its registers hold (28 at 72 registers, 24 at
-// 80); 1 = no split.
+// the pixels within the warps its registers hold (FP32: 28 at 72 registers,
+// 24 at 80; FP64: 16 at 128); 1 = no split.  FP64 takes a power of two, so
+// that the shares divide evenly.
 inline int ga_segments(int npix, int npop, int nl, int regs)
 {
-    const int warps = regs <= 72 ? 28 : 24, per_sm = (npix + 151) / 152;
+    const int warps = regs <= 72 ? 28 : regs <= 80 ? 24 : 16, per_sm = (npix + 151) / 152;
     const int s = warps / (per_sm * (npop / 32)), npair = (nl + 1) / 2;
+    if (regs > 80) return s >= 8 ? 8 : s >= 4 ? 4 : s >= 2 ? 2 : 1;
     return s < npair ? s : npair;
 }
 
@@ -766,8 +785,9 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
                             KSub sub = {})
 {
     const int nlines = NL > 0 ? NL : pb.n_lines;
-    if constexpr (sizeof(R) == 4 && MAXT <= 256 && !COUNT) {
-        const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, NL > 0 && !PAT ? GENESIS_GA_NREG32 : 80);
+    if constexpr (MAXT <= 256 && !COUNT) {
+        const int regs = sizeof(R) == 8 ? 128 : NL > 0 && !PAT ? GENESIS_GA_NREG32 : 80;
+        const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, regs);
         const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M, true);
         if (nseg > 1 && L.total <= 200 * 1024) {
             auto kern = k_ga_evolve<R, NL, MAXT, false, PAT, M, true>;

@@ -10,7 +10,7 @@
 //    0.3125 in |x|; w(-x + i a) is the conjugate): 29 operations instead of
 //    the 105 of Weideman's series.  The 32 lanes of one warp build the table,
 //    a cell each: w at the centre from the Taylor coefficients of the nearest
-//    node of a fixed grid (faddeeva_nodes.h; a step along i of at most 0.078)
+//    node of a fixed grid (faddeeva_nodes.h; a step along i of at most 0.04)
 //    and the further coefficients by c_{n+1} = -2 (z c_n + c_{n-1}) / (n + 1)
 //    (from w' = -2 z w + 2 i / sqrt(pi)).  The first omitted term is below
 //    6e-17.  Measured against 40-digit values the table is within 2e-16 of w;
@@ -114,6 +114,9 @@ struct ExtTable {
 };
 static __device__ const ExtTable d_ext{};
 
+// First row and first coefficient of the K-th convergent in ExtTable's order.
+template <int K> constexpr int kExtFirst = K == 5 ? 0 : K == 7 ? 18 : 42;
+
 // Everything a block holds for one model.
 struct ProfShared {
     double2 cell[kCells * (kTaylor + 1)];  // Taylor coefficients (re, im) of a cell, ascending
@@ -150,7 +153,7 @@ __device__ __forceinline__ void build_cells(ProfShared &S, const double2 *nodes,
     C2<double> m;
     if (y >= 0.0) {  // from the node at x and the nearest y: a step along i
         const int iy = min((int)(narrow(y) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
-        const double2 *c = nodes + ((size_t)iy * kNodeGrid + 2 * lane + 1) * kNodeCoef;
+        const double2 *c = nodes + ((size_t)iy * kNodeGrid + 4 * lane + 2) * kNodeCoef;
         const double dy = y - widen((float)iy * (float)kNodeStep);
         const double2 top = __ldg(c + kNodeCoef - 1);
         m = {top.x, top.y};

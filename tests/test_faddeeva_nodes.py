@@ -8,7 +8,7 @@ import pytest
 
 scipy_special = pytest.importorskip("scipy.special")
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1208_0302_gb300", "csrc")
-N, H, TERMS = 65, 0.15625, 14
+N, H, TERMS = 129, 0.078125, 11
 
 
 @pytest.fixture(scope="module")
@@ -34,7 +34,7 @@ def test_node_values(nodes):
 
 @pytest.mark.parametrize("dx,dy", [(0.5, 0.5), (-0.5, 0.5), (0.5, -0.5), (0.0, 0.5)])
 def test_expansions_reach_the_cell(nodes, dx, dy):
-    # 14 terms: the first omitted is below (0.11)^14 / Gamma(8) = 8e-18
+    # 11 terms: the first omitted is below (0.0553)^11 / Gamma(6.5) = 5e-17
     iy, ix = np.mgrid[1:N - 1, 1:N - 1]
     dz = H * (dx + 1j * dy)
     s = np.zeros(ix.shape, dtype=complex)
