@@ -461,7 +461,7 @@ cudaError_t classify_t(const KProblem &pb, const void *obs, int npix, const KCla
 {
     const int smem = pb.n_lambda * (int)sizeof(GridTables) + ROLES * 4 * 32 * kPitch * (int)sizeof(RO);
     auto kern = k_classify<RO, ROLES>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(npix + 31) / 32, 32 * ROLES, smem, st>>>(pb, (const RO *)obs, npix, c);
     return cudaGetLastError();

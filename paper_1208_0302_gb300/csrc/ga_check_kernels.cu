@@ -81,7 +81,7 @@ cudaError_t launch_fitness_t(const KProblem &pb, int weight_mode, const void *ob
     const int nlines = NL > 0 ? NL : pb.n_lines;
     const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, npop, M);
     auto kern = k_ga_fitness<R, NL, MAXT, PAT, M>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+    cudaError_t e = allow_smem(kern, L.total);
     if (e != cudaSuccess) return e;
     kern<<<npix, npop, L.total, st>>>(pb, weight_mode, (const R *)obs, w, mu_px, nactive, params, fit, (R *)res);
     return cudaGetLastError();

@@ -791,7 +791,7 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
         const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M, true);
         if (nseg > 1 && L.total <= 200 * 1024) {
             auto kern = k_ga_evolve<R, NL, MAXT, false, PAT, M, true>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+            cudaError_t e = allow_smem(kern, L.total);
             if (e != cudaSuccess) return e;
             kern<<<npix, nseg * ga.npop, L.total, st>>>(pb, ga, (const R *)obs, w, mu_px, npix, best, best_genes,
                                                         counts, sd, sub);
@@ -800,7 +800,7 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
     }
     const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M);
     auto kern = k_ga_evolve<R, NL, MAXT, COUNT, PAT, M, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, L.total);
+    cudaError_t e = allow_smem(kern, L.total);
     if (e != cudaSuccess) return e;
     kern<<<npix, ga.npop, L.total, st>>>(pb, ga, (const R *)obs, w, mu_px, npix, best, best_genes, counts,
                                           sd, sub);

@@ -9,6 +9,14 @@
 
 namespace genesis {
 
+// Let a kernel take `bytes` of dynamic shared memory (only above the 48 KB
+// that every kernel may have is a call to the runtime needed).
+template <class Kernel> inline cudaError_t allow_smem(Kernel kern, size_t bytes)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 // GA launch parameters (Section 3 operators, Section 5.6 restarts).
 struct KGa {
     int npop, ngen, nsamp, weight_mode;

@@ -444,7 +444,7 @@ cudaError_t sigma_t(const KProblem &pb, const void *obs, const double *w, const 
     const int nlines = NL > 0 ? NL : pb.n_lines;
     const size_t smem = sizeof(LmWarpSmem<R>) * kLmWarps + sizeof(R) * (ME_MAX_LINES + (size_t)nlines * pb.n_lambda);
     auto kern = k_lm_sigma<R, RO, NL, M>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(npix + kLmWarps - 1) / kLmWarps, kLmWarps * 32, smem, st>>>(pb, (const RO *)obs, w, mu_px, npix,
                                                                        params, sigma);
@@ -458,7 +458,7 @@ cudaError_t lm_t(const KProblem &pb, const KLm &lm, const void *obs, const doubl
     const int nlines = NL > 0 ? NL : pb.n_lines;
     const size_t smem = sizeof(LmWarpSmem<R>) * kLmWarps + sizeof(R) * (ME_MAX_LINES + (size_t)nlines * pb.n_lambda);
     auto kern = k_lm<R, RO, NL, M>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(npix + kLmWarps - 1) / kLmWarps, kLmWarps * 32, smem, st>>>(pb, lm, (const RO *)obs, w, mu_px,
                                                                       npix, params, sub);

@@ -1,4 +1,7 @@
 // Stokes synthesis, Jacobian, adjoint and FP64 chi-square kernels (sm_103a).
+#include <algorithm>
+#include <type_traits>
+
 #include "async_copy.cuh"
 #include "kernels.h"
 #include "me_jac.cuh"
@@ -39,82 +42,94 @@ __device__ __forceinline__ void stage_offsets(const KProblem &pb, int nlines, R 
         s_he[threadIdx.x] = threadIdx.x < nlines ? R(pb.line[threadIdx.x].half_eta) : R(0);
 }
 
-// One thread per (model, wavelength).
-template <class R, int NL, bool FILL = false>
-__global__ void __launch_bounds__(kSynthBlock)
-k_synth(const __grid_constant__ KProblem pb, const double *__restrict__ params,
-        const double *__restrict__ mu_px, int n, R *__restrict__ stokes)
+// A model's parameters (and mu) on every lane in the problem's precision: one
+// lane loads and converts each (conversions take the FP64 pipe, a warp
+// instruction in 16 clocks of an SM), shuffles spread them.
+template <class R, int M>
+__device__ __forceinline__ void load_model(const KProblem &pb, const double *params, const double *mu_px, int m, R (&p)[M],
+                                           R &mu)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int nl = pb.n_lambda, nlines = NL > 0 ? NL : pb.n_lines;
-    R *s_he = (R *)smem;
-    R *s_doff = s_he + ME_MAX_LINES;
-    stage_offsets<R>(pb, nlines, s_doff, s_he);
-    __syncthreads();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)n * nl) return;
-    const int m = (int)(i / nl), j = (int)(i - (long long)m * nl);
-    constexpr int M = kNpar<FILL>;
-    R p[M];
+    const int lane = threadIdx.x & 31;
+    const double v = lane < M ? params[(size_t)m * M + lane] : mu_px ? mu_px[m] : pb.mu;
+    const R r = R(v);
 #pragma unroll
-    for (int d = 0; d < M; ++d) p[d] = R(params[(size_t)m * M + d]);
-    const R mu = mu_px ? R(mu_px[m]) : R(pb.mu);
-    const Geo<R> g = make_geo<R, NL, FILL>(pb, nlines, p, mu);
-    R doff[ME_MAX_LINES], he[ME_MAX_LINES];
-#pragma unroll
-    for (int l = 0; l < ME_MAX_LINES; ++l) {
-        doff[l] = l < nlines ? s_doff[l * nl + j] : R(0);
-        he[l] = s_he[l];
-    }
-    const Stokes4<R> s = me_point<R, NL, true, FILL>(g, doff, he, nlines, pb.line);
-    R *o = stokes + (size_t)m * 4 * nl;
-    o[j] = s.I;
-    o[nl + j] = s.Q;
-    o[2 * nl + j] = s.U;
-    o[3 * nl + j] = s.V;
+    for (int d = 0; d < M; ++d) p[d] = __shfl_sync(0xffffffffu, r, d);
+    mu = __shfl_sync(0xffffffffu, r, M);
 }
 
-template <class R, int NL, bool FILL = false>
-__global__ void __launch_bounds__(kSynthBlock)
-k_jac(const __grid_constant__ KProblem pb, const double *__restrict__ params,
-      const double *__restrict__ mu_px, int n, R *__restrict__ stokes, R *__restrict__ jac)
+// Blocks per SM that the FP32 Jacobian's registers have to allow: 20 011
+// two-line models take 145, 128, 227 and 255 us at 3, 4, 5 and 6.
+constexpr int kJacMinB = 4;
+
+// Synthesis, and with JAC the Jacobian, a warp per model (or per `per` of its
+// chunks of 32 wavelengths, while there are too few models to fill the chip):
+// lanes over wavelengths, the model's geometry formed once for the warp's
+// chunks, the wavelength offsets once for all of a block's models.  A thread
+// per (model, wavelength) formed both for every point: ten FP64 conversions
+// per warp alone took longer than the synthesis.  A Jacobian row of Stokes s
+// and 32 wavelengths leaves through shared memory as 32 M consecutive values,
+// so that each store instruction writes whole sectors (lane by lane it wrote
+// 4 of every 36 bytes).  20 011 two-line FP32 models, 128 wavelengths:
+// syntheses 110 -> 55 us, Jacobians 267 -> 128 us.
+template <class R, int NL, bool FILL, bool JAC>
+__global__ void __launch_bounds__(kSynthBlock, sizeof(R) == 8 ? 1 : JAC ? kJacMinB : 8)
+k_models(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
+         int n, int per, R *__restrict__ stokes, R *__restrict__ jac)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int M = kNpar<FILL>;
     const int nl = pb.n_lambda, nlines = NL > 0 ? NL : pb.n_lines;
     R *s_he = (R *)smem;
     R *s_doff = s_he + ME_MAX_LINES;
     stage_offsets<R>(pb, nlines, s_doff, s_he);
     __syncthreads();
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (long long)n * nl) return;
-    const int m = (int)(i / nl), j = (int)(i - (long long)m * nl);
-    constexpr int M = kNpar<FILL>;
-    R p[M];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    R *s_row = s_doff + nlines * nl + warp * 32 * M;
+    R he[ME_MAX_LINES];
 #pragma unroll
-    for (int d = 0; d < M; ++d) p[d] = R(params[(size_t)m * M + d]);
-    const R mu = mu_px ? R(mu_px[m]) : R(pb.mu);
-    const GeoJ<R> G = make_geoj<R, NL, FILL>(pb, nlines, p, mu);
-    R doff[ME_MAX_LINES], he[ME_MAX_LINES];
+    for (int l = 0; l < ME_MAX_LINES; ++l) he[l] = s_he[l];
+    const int chunks = (nl + 31) >> 5, groups = (chunks + per - 1) / per;
+    const long long items = (long long)n * groups;
+    for (long long it = (long long)blockIdx.x * (kSynthBlock / 32) + warp; it < items;
+         it += (long long)gridDim.x * (kSynthBlock / 32)) {
+        const int m = (int)(it / groups), c0 = (int)(it - (long long)m * groups) * per;
+        R p[M], mu;
+        load_model<R, M>(pb, params, mu_px, m, p, mu);
+        std::conditional_t<JAC, GeoJ<R>, Geo<R>> G;
+        if constexpr (JAC) G = make_geoj<R, NL, FILL>(pb, nlines, p, mu);
+        else G = make_geo<R, NL, FILL>(pb, nlines, p, mu);
+        for (int c = c0; c < min(c0 + per, chunks); ++c) {
+            const int j = c * 32 + lane;
+            const bool on = j < nl;
+            R doff[ME_MAX_LINES];
 #pragma unroll
-    for (int l = 0; l < ME_MAX_LINES; ++l) {
-        doff[l] = l < nlines ? s_doff[l * nl + j] : R(0);
-        he[l] = s_he[l];
-    }
-    Stokes4<R> s;
-    R J[4][M];
-    me_point_jac<R, NL, FILL>(G, doff, he, nlines, pb.line, s, J);
-    if (stokes) {
-        R *o = stokes + (size_t)m * 4 * nl;
-        o[j] = s.I;
-        o[nl + j] = s.Q;
-        o[2 * nl + j] = s.U;
-        o[3 * nl + j] = s.V;
-    }
+            for (int l = 0; l < ME_MAX_LINES; ++l) doff[l] = l < nlines ? s_doff[l * nl + (on ? j : nl - 1)] : R(0);
+            Stokes4<R> s;
+            R J[4][M];
+            if constexpr (JAC) me_point_jac<R, NL, FILL>(G, doff, he, nlines, pb.line, s, J);
+            else s = me_point<R, NL, true, FILL>(G, doff, he, nlines, pb.line);
+            if (stokes && on) {
+                R *o = stokes + (size_t)m * 4 * nl + j;
+                o[0] = s.I;
+                o[nl] = s.Q;
+                o[2 * nl] = s.U;
+                o[3 * nl] = s.V;
+            }
+            if constexpr (JAC) {
+                const int len = min(32, nl - c * 32) * M;
 #pragma unroll
-    for (int st = 0; st < 4; ++st) {
-        R *o = jac + (((size_t)m * 4 + st) * nl + j) * M;
+                for (int st = 0; st < 4; ++st) {
 #pragma unroll
-        for (int k = 0; k < M; ++k) o[k] = J[st][k];
+                    for (int k = 0; k < M; ++k) s_row[lane * M + k] = J[st][k];
+                    __syncwarp();
+                    R *o = jac + (((size_t)m * 4 + st) * nl + c * 32) * M;
+#pragma unroll
+                    for (int k = 0; k < M; ++k)
+                        if (k * 32 + lane < len) o[k * 32 + lane] = s_row[k * 32 + lane];
+                    __syncwarp();
+                }
+            }
+        }
     }
 }
 
@@ -421,13 +436,21 @@ template <class R> size_t offsets_smem(const KProblem &pb)
     return sizeof(R) * (ME_MAX_LINES + (size_t)pb.n_lines * pb.n_lambda);
 }
 
-template <class R, int NL, bool FILL = false>
-cudaError_t synth_t(const KProblem &pb, const double *params, const double *mu_px, int n,
-                    void *stokes, cudaStream_t st)
+template <class R, int NL, bool FILL, bool JAC>
+cudaError_t models_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes, void *jac,
+                     cudaStream_t st)
 {
-    const long long tot = (long long)n * pb.n_lambda;
-    const int blocks = (int)((tot + kSynthBlock - 1) / kSynthBlock);
-    k_synth<R, NL, FILL><<<blocks, kSynthBlock, offsets_smem<R>(pb), st>>>(pb, params, mu_px, n, (R *)stokes);
+    constexpr int kWarps = kSynthBlock / 32;
+    const int chunks = (pb.n_lambda + 31) / 32;
+    // a warp takes a whole model once the models alone give an SM 16 warps
+    const int per = n >= 152 * 16 ? chunks : 1;
+    const long long items = (long long)n * ((chunks + per - 1) / per);
+    const long long blocks = std::min((items + kWarps - 1) / kWarps, (long long)152 * (JAC ? 8 : 16));
+    const size_t smem = offsets_smem<R>(pb) + (JAC ? sizeof(R) * kWarps * 32 * kNpar<FILL> : 0);
+    auto kern = k_models<R, NL, FILL, JAC>;
+    cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(int)blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, per, (R *)stokes, (R *)jac);
     return cudaGetLastError();
 }
 
@@ -437,20 +460,9 @@ cudaError_t synth64_t(const KProblem &pb, const double *params, const double *mu
 {
     auto kern = k_synth64<FILL>;
     const size_t smem = prof_smem(pb);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<n, kProfBlock, smem, st>>>(pb, params, mu_px, (double *)stokes);
-    return cudaGetLastError();
-}
-
-template <class R, int NL, bool FILL = false>
-cudaError_t jac_t(const KProblem &pb, const double *params, const double *mu_px, int n,
-                  void *stokes, void *jac, cudaStream_t st)
-{
-    const long long tot = (long long)n * pb.n_lambda;
-    const int blocks = (int)((tot + kSynthBlock - 1) / kSynthBlock);
-    k_jac<R, NL, FILL><<<blocks, kSynthBlock, offsets_smem<R>(pb), st>>>(pb, params, mu_px, n, (R *)stokes,
-                                                                  (R *)jac);
     return cudaGetLastError();
 }
 
@@ -473,10 +485,10 @@ cudaError_t launch_synth(const KProblem &pb, int dtype, const double *params, co
     if (dtype != ME_F32)
         return pb.fill ? synth64_t<true>(pb, params, mu_px, n, stokes, st)
                        : synth64_t<false>(pb, params, mu_px, n, stokes, st);
-    if (pb.fill) return synth_t<float, 0, true>(pb, params, mu_px, n, stokes, st);
-    if (pb.n_lines == 1) return synth_t<float, 1>(pb, params, mu_px, n, stokes, st);
-    if (pb.n_lines == 2) return synth_t<float, 2>(pb, params, mu_px, n, stokes, st);
-    return synth_t<float, 0>(pb, params, mu_px, n, stokes, st);
+    if (pb.fill) return models_t<float, 0, true, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    if (pb.n_lines == 1) return models_t<float, 1, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    if (pb.n_lines == 2) return models_t<float, 2, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    return models_t<float, 0, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
 }
 
 cudaError_t launch_jac(const KProblem &pb, int dtype, const double *params, const double *mu_px,
@@ -484,14 +496,14 @@ cudaError_t launch_jac(const KProblem &pb, int dtype, const double *params, cons
 {
     if (n <= 0) return cudaSuccess;
     if (pb.fill)
-        return dtype == ME_F32 ? jac_t<float, 0, true>(pb, params, mu_px, n, stokes, jac, st)
-                               : jac_t<double, 0, true>(pb, params, mu_px, n, stokes, jac, st);
+        return dtype == ME_F32 ? models_t<float, 0, true, true>(pb, params, mu_px, n, stokes, jac, st)
+                               : models_t<double, 0, true, true>(pb, params, mu_px, n, stokes, jac, st);
     if (dtype == ME_F32) {
-        if (pb.n_lines == 1) return jac_t<float, 1>(pb, params, mu_px, n, stokes, jac, st);
-        if (pb.n_lines == 2) return jac_t<float, 2>(pb, params, mu_px, n, stokes, jac, st);
-        return jac_t<float, 0>(pb, params, mu_px, n, stokes, jac, st);
+        if (pb.n_lines == 1) return models_t<float, 1, false, true>(pb, params, mu_px, n, stokes, jac, st);
+        if (pb.n_lines == 2) return models_t<float, 2, false, true>(pb, params, mu_px, n, stokes, jac, st);
+        return models_t<float, 0, false, true>(pb, params, mu_px, n, stokes, jac, st);
     }
-    return jac_t<double, 0>(pb, params, mu_px, n, stokes, jac, st);
+    return models_t<double, 0, false, true>(pb, params, mu_px, n, stokes, jac, st);
 }
 
 cudaError_t launch_vjp(const KProblem &pb, int dtype, const double *params, const double *mu_px,
@@ -518,7 +530,7 @@ cudaError_t line_centre_t(const KProblem &pb, const void *obs, int npix, int W, 
     constexpr int PIX = 32 / G;
     const int smem = lo <= hi ? PIX * ((hi - lo + 2 * W + 1) | 1) * (sizeof(RO) == 4 ? 12 : 8) : 0;
     auto kern = k_line_centre<RO, G>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(npix + PIX - 1) / PIX, 32, smem, st>>>(pb, (const RO *)obs, npix, W, lo, hi, lam_c, idx);
     return cudaGetLastError();
@@ -554,7 +566,7 @@ static cudaError_t chi2_t(const KProblem &pb, const void *obs, const double *w, 
 {
     auto kern = k_chi2_f64<RO, FILL>;
     const size_t smem = prof_smem(pb);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<npix, kProfBlock, smem, st>>>(pb, (const RO *)obs, w, mu_px, npix, params, chi2, sub);
     return cudaGetLastError();
