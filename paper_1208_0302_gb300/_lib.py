@@ -137,6 +137,8 @@ def library_path() -> str:
 def load(build_if_missing: bool = True):
     """Load libgenesis.so (building it first if asked and needed)."""
     global _lib
+    if _lib is not None:  # set once, complete
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib

