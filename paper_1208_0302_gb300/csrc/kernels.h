@@ -9,11 +9,12 @@
 
 namespace genesis {
 
-// Let a kernel take `bytes` of dynamic shared memory (only above the 48 KB
-// that every kernel may have is a call to the runtime needed).
+// Let a kernel take `bytes` of dynamic shared memory.  A call to the runtime
+// is needed only above the 48 KB that every kernel may have, static arrays (at
+// most 8 KB here) included.
 template <class Kernel> inline cudaError_t allow_smem(Kernel kern, size_t bytes)
 {
-    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes <= 40 * 1024) return cudaSuccess;
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 

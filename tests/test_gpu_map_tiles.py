@@ -16,7 +16,8 @@ def _tile(a, n):
 
 
 @pytest.mark.parametrize("dtype,nl,npix", [("f32", 97, 31), ("f32", 128, 33), ("f64", 45, 64), ("f32", 128, 9728),
-                                           ("f32", 131, 9729), ("f64", 96, 9761)])
+                                           ("f32", 131, 9729), ("f64", 96, 9761),
+                                           ("f32", 340, 40)])
 def test_classify_launch_shapes(gpu, orc, dtype, nl, npix):
     spec = gi.two_line_spec(nl)
     _, obs = make_obs(orc, spec, min(npix, 61), seed=nl)
