@@ -310,14 +310,25 @@ template <class R> __device__ __forceinline__ int stable_rank(const R *s_fit, in
     return r;
 }
 
+// KGa's mutation thresholds in shared memory, where lanes read different
+// entries at once: row b holds t(b, 0..b), then zeros (nothing is below them).
+__device__ __forceinline__ void stage_thresholds(const KGa &ga, uint64_t *s_tmut)
+{
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+        const int b = i >> 4, c = i & 15;
+        s_tmut[i] = c <= b ? ga.t_mut[b * (b + 1) / 2 + c] : 0;
+    }
+}
+
 // Select (binary tournament), recombine (one-point crossover with lane k^1),
-// mutate (per-bit, LSB-biased) and elitism for child slot k.  t_mut: KGa's
-// thresholds in shared memory, where lanes read different entries at once.
+// mutate (per-bit, LSB-biased) and elitism for child slot k.  t_mut: the
+// thresholds of stage_thresholds; s_draw: this slot's 16 draws, npop apart.
 // Must be called by all lanes of full warps (npop is a multiple of 32).
 template <class R, int M>
 __device__ __forceinline__ void breed_one(const KGa &ga, uint64_t pid, int t, int k, int npop,
                                           const R *s_fit, const uint16_t *s_cur, int elite,
-                                          const uint64_t *t_mut, uint16_t *s_row, uint16_t g[M])
+                                          const uint64_t *t_mut, uint32_t *s_draw, uint16_t *s_row,
+                                          uint16_t g[M])
 {
     const U4 u = ga_random_rk(ga.rk, pid, t, (uint32_t)k, kPurposeSelect);
     const int i = (int)(((uint64_t)u.x * (uint64_t)npop) >> 32);
@@ -353,34 +364,47 @@ __device__ __forceinline__ void breed_one(const KGa &ga, uint64_t pid, int t, in
     // from the word's LSB toward its MSB: with bits 0..b still open, u >=
     // t(b, 0) leaves them all unflipped; otherwise the next flip is bit c, the
     // largest c <= b with u < t(b, c), and bits 0..c-1 stay open.  A word
-    // without flips takes one draw.  The loop runs over draws, not words: the
-    // lanes of a warp use one draw each per turn, so blocks are generated by
-    // all lanes at once and a warp takes as many turns as its busiest lane has
-    // draws (about 14 for M = 9, where word by word it took two or three turns
-    // in each word); lanes search different rows, which shared memory serves
-    // in parallel and the constant bank one address at a time.  Two-line GA,
-    // 16 384 pixels, population 128, 100 generations: 164.9 -> 159.8 ms.
+    // without flips takes one draw.  Sixteen draws (four independent blocks)
+    // are made at once, enough for nearly every slot, with a mask of those
+    // that flip a bit of a fresh word; the mask skips the words without flips,
+    // so a warp loops over its busiest lane's flips and not over its draws.  c
+    // takes two rounds of three independent threshold reads.  Two-line GA, 16
+    // 384 pixels, population 128, 30 generations: 64.1 -> 62.6 ms; 64 pixels,
+    // population 64, 100 generations: 1.57 -> 1.40 ms.
 #pragma unroll
     for (int d = 0; d < M; ++d) s_row[d] = g[d];
+    const uint64_t t0 = ga.t_mut[120];  // t(15, 0)
     int word = 0, b = 15;
-    for (uint32_t nblk = 0; __any_sync(0xffffffffu, word < M); ++nblk) {
-        const U4 blk = ga_random_rk(ga.rk, pid, t, (uint32_t)k, kPurposeMutate + nblk);
+    for (uint32_t blk = 0; __any_sync(0xffffffffu, word < M); blk += 4) {
+        uint32_t flips = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            if (word >= M) continue;
-            const uint64_t uv = e == 0 ? blk.x : e == 1 ? blk.y : e == 2 ? blk.z : blk.w;
-            const uint64_t *row = t_mut + b * (b + 1) / 2;
-            int c = 0;
-            if (uv < row[0]) {
-                int hi = b;  // the largest c with uv < row[c]; row[0] qualifies
-                while (c < hi) {
-                    const int mid = (c + hi + 1) >> 1;
-                    if (uv < row[mid]) c = mid;
-                    else hi = mid - 1;
-                }
-                s_row[word] ^= (uint16_t)(1u << (15 - c));
+            const U4 r = ga_random_rk(ga.rk, pid, t, (uint32_t)k, kPurposeMutate + blk + e);
+            s_draw[(4 * e) * npop] = r.x;
+            s_draw[(4 * e + 1) * npop] = r.y;
+            s_draw[(4 * e + 2) * npop] = r.z;
+            s_draw[(4 * e + 3) * npop] = r.w;
+            flips |= ((r.x < t0 ? 1u : 0u) | (r.y < t0 ? 2u : 0u) | (r.z < t0 ? 4u : 0u) | (r.w < t0 ? 8u : 0u)) << (4 * e);
+        }
+        int i = 0;
+        while (word < M && i < 16) {
+            if (b == 15) {
+                const uint32_t rest = flips >> i;
+                const int skip = min(rest ? __ffs(rest) - 1 : 16 - i, M - word);
+                word += skip;
+                i += skip;
+                if (word >= M || i >= 16) break;
             }
-            b = c - 1;  // no flip: as after a flip of bit 0
+            const uint64_t u = s_draw[i * npop], *row = t_mut + 16 * b;
+            ++i;
+            const int q = 4 * ((u < row[4] ? 1 : 0) + (u < row[8] ? 1 : 0) + (u < row[12] ? 1 : 0));
+            const int c = q + (u < row[q + 1] ? 1 : 0) + (u < row[q + 2] ? 1 : 0) + (u < row[q + 3] ? 1 : 0);
+            if (u < row[0]) {
+                s_row[word] ^= (uint16_t)(1u << (15 - c));
+                b = c - 1;
+            } else {
+                b = -1;
+            }
             if (b < 0) {
                 b = 15;
                 ++word;
@@ -420,9 +444,10 @@ __host__ __device__ __forceinline__ GaSmem ga_smem_layout(int nl, int nlines, in
     L.w2 = take(8 * (int)sizeof(R), 16);  // w^2 of I, Q, U, V, then w
     L.he = take(4 * (int)sizeof(R), 16);
     L.dom = take((int)sizeof(DecodeDomain), 16);  // the pixel's decode domain
-    L.tmut = take(136 * 8, 16);                   // mutation thresholds
+    L.tmut = take(256 * 8, 16);                   // mutation thresholds
     L.genes = take(2 * npop * npar * 2, 16);
-    L.kc = take(sizeof(R) == 4 ? 3 * npop * 16 : 0, 16);  // FP32: 3 float4 of closed-form constants per thread
+    // 16 mutation draws per thread; FP32: then 3 float4 of closed-form constants
+    L.kc = take(16 * npop * 4, 16);
     L.part = take(sizeof(R) == 4 && split ? (nl + 1) / 2 * npop * 4 : 0, 16);  // FP32: a split block's pair sums
     L.f64 = take(sizeof(R) == 8 && npop <= 256 ? fit64_doubles(npop) * 8 : 0, 16);  // FP64: see Fit64Shared
     L.total = (o + 15) / 16 * 16;
@@ -611,7 +636,7 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     // per-launch constants
     const R inv_nu = R(1) / R(4 * nl - M);
     stage_offsets_ga<R>(pb, nlines, nl, tid, s_doff, s_he);
-    for (int i = tid; i < 136; i += blockDim.x) s_tmut[i] = ga.t_mut[i];
+    stage_thresholds(ga, s_tmut);
 
     const int nrun = sub.count ? min(*sub.count, npix) : npix;
     for (int blk = blockIdx.x; blk < nrun; blk += gridDim.x) {
@@ -695,7 +720,8 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
             const uint16_t *s_cur = s_genes + cur * npop * M;
             uint16_t *s_nxt = s_genes + (cur ^ 1) * npop * M;
             if (seg == 0) {
-                breed_one<R, M>(ga, pid, t, k, npop, s_fit, s_cur, elite, s_tmut, s_nxt + k * M, g);  // a10-a12
+                breed_one<R, M>(ga, pid, t, k, npop, s_fit, s_cur, elite, s_tmut, (uint32_t *)s_kc + k,
+                                s_nxt + k * M, g);  // a10-a12
                 if (SPLIT) {
 #pragma unroll
                     for (int d = 0; d < M; ++d) s_nxt[k * M + d] = g[d];

@@ -34,8 +34,9 @@ __global__ void k_ga_breed(const __grid_constant__ KGa ga, const uint16_t *__res
     int *s_widx = (int *)(s_wmin + 32);
     uint16_t *s_cur = (uint16_t *)(s_widx + 32);
     uint16_t *s_new = s_cur + npop * M;
-    __shared__ uint64_t s_tmut[136];
-    for (int i = k; i < 136; i += npop) s_tmut[i] = ga.t_mut[i];
+    uint32_t *s_draw = (uint32_t *)(smem + (npop * 8 + 32 * 8 + 32 * 4 + 2 * npop * M * 2));
+    __shared__ uint64_t s_tmut[256];
+    stage_thresholds(ga, s_tmut);
     const size_t base = (size_t)prob * npop;
     s_fit[k] = clean_fit(fit[base + k]);
 #pragma unroll
@@ -44,7 +45,7 @@ __global__ void k_ga_breed(const __grid_constant__ KGa ga, const uint16_t *__res
     const int elite = block_argmin<double>(s_fit, npop, s_wmin, s_widx);
     uint16_t g[M];
     breed_one<double, M>(ga, ga.pixel_id0 + (uint64_t)prob, gen, k, npop, s_fit, s_cur, elite,
-                      s_tmut, s_new + k * M, g);
+                      s_tmut, s_draw + k, s_new + k * M, g);
 #pragma unroll
     for (int d = 0; d < M; ++d) child[(base + k) * M + d] = g[d];
     if (k == 0 && elite_out) elite_out[prob] = elite;
@@ -143,7 +144,9 @@ cudaError_t launch_ga_breed(const KGa &ga, int npar, const uint16_t *genes, cons
                             int gen, uint16_t *child, int *elite, cudaStream_t st)
 {
     if (nprob <= 0) return cudaSuccess;
-    const int smem = ga.npop * 8 + 32 * 8 + 32 * 4 + 2 * ga.npop * npar * 2;
+    const int smem = ga.npop * 8 + 32 * 8 + 32 * 4 + 2 * ga.npop * npar * 2 + 16 * ga.npop * 4;
+    cudaError_t e = npar == ME_NPAR_MAX ? allow_smem(k_ga_breed<ME_NPAR_MAX>, smem) : allow_smem(k_ga_breed<ME_NPAR>, smem);
+    if (e != cudaSuccess) return e;
     if (npar == ME_NPAR_MAX)
         k_ga_breed<ME_NPAR_MAX><<<nprob, ga.npop, smem, st>>>(ga, genes, fit, gen, child, elite);
     else
