@@ -62,7 +62,7 @@ __device__ __forceinline__ void load_model(const KProblem &pb, const double *par
 constexpr int kJacMinB = 4;
 
 // Synthesis, and with JAC the Jacobian, a warp per model (or per `per` of its
-// chunks of 32 wavelengths, while there are too few models to fill the chip):
+// chunks of 32 wavelengths, where whole models would leave warps idle):
 // lanes over wavelengths, the model's geometry formed once for the warp's
 // chunks, the wavelength offsets once for all of a block's models.  A thread
 // per (model, wavelength) formed both for every point: ten FP64 conversions
@@ -71,11 +71,12 @@ constexpr int kJacMinB = 4;
 // so that each store instruction writes whole sectors (lane by lane it wrote
 // 4 of every 36 bytes).  20 011 two-line FP32 models, 128 wavelengths:
 // syntheses 110 -> 55 us, Jacobians 267 -> 128 us.
-template <class R, int NL, bool FILL, bool JAC>
-__global__ void __launch_bounds__(kSynthBlock, sizeof(R) == 8 ? 1 : JAC ? kJacMinB : 8)
+template <int NL, bool FILL, bool JAC>
+__global__ void __launch_bounds__(kSynthBlock, JAC ? kJacMinB : 8)
 k_models(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
-         int n, int per, R *__restrict__ stokes, R *__restrict__ jac)
+         int n, int per, float *__restrict__ stokes, float *__restrict__ jac)
 {
+    using R = float;
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int M = kNpar<FILL>;
     const int nl = pb.n_lambda, nlines = NL > 0 ? NL : pb.n_lines;
@@ -130,6 +131,53 @@ k_models(const __grid_constant__ KProblem pb, const double *__restrict__ params,
                 }
             }
         }
+    }
+}
+
+// FP64 Jacobian, one thread per (model, wavelength): bound by the FP64 pipe,
+// where the warp-per-model form above was 0 to 5 % slower (700 full-pattern
+// models 556 against 525 us).
+template <bool FILL>
+__global__ void __launch_bounds__(kSynthBlock)
+k_jac64(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px, int n,
+        double *__restrict__ stokes, double *__restrict__ jac)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int nl = pb.n_lambda, nlines = pb.n_lines;
+    double *s_he = (double *)smem;
+    double *s_doff = s_he + ME_MAX_LINES;
+    stage_offsets<double>(pb, nlines, s_doff, s_he);
+    __syncthreads();
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (long long)n * nl) return;
+    const int m = (int)(i / nl), j = (int)(i - (long long)m * nl);
+    constexpr int M = kNpar<FILL>;
+    double p[M];
+#pragma unroll
+    for (int d = 0; d < M; ++d) p[d] = params[(size_t)m * M + d];
+    const double mu = mu_px ? mu_px[m] : pb.mu;
+    const GeoJ<double> G = make_geoj<double, 0, FILL>(pb, nlines, p, mu);
+    double doff[ME_MAX_LINES], he[ME_MAX_LINES];
+#pragma unroll
+    for (int l = 0; l < ME_MAX_LINES; ++l) {
+        doff[l] = l < nlines ? s_doff[l * nl + j] : 0.0;
+        he[l] = s_he[l];
+    }
+    Stokes4<double> s;
+    double J[4][M];
+    me_point_jac<double, 0, FILL>(G, doff, he, nlines, pb.line, s, J);
+    if (stokes) {
+        double *o = stokes + (size_t)m * 4 * nl;
+        o[j] = s.I;
+        o[nl + j] = s.Q;
+        o[2 * nl + j] = s.U;
+        o[3 * nl + j] = s.V;
+    }
+#pragma unroll
+    for (int st = 0; st < 4; ++st) {
+        double *o = jac + (((size_t)m * 4 + st) * nl + j) * M;
+#pragma unroll
+        for (int k = 0; k < M; ++k) o[k] = J[st][k];
     }
 }
 
@@ -436,21 +484,32 @@ template <class R> size_t offsets_smem(const KProblem &pb)
     return sizeof(R) * (ME_MAX_LINES + (size_t)pb.n_lines * pb.n_lambda);
 }
 
-template <class R, int NL, bool FILL, bool JAC>
+template <int NL, bool FILL, bool JAC>
 cudaError_t models_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes, void *jac,
                      cudaStream_t st)
 {
     constexpr int kWarps = kSynthBlock / 32;
+    // resident warps, and a model's geometry in units of a chunk's work
+    const int resident = 152 * (JAC ? kJacMinB : 8) * kWarps;
+    const double geometry = JAC ? 0.2 : 0.8;
     const int chunks = (pb.n_lambda + 31) / 32;
-    // a warp takes a whole model once the models alone give an SM 16 warps
-    const int per = n >= 152 * 16 ? chunks : 1;
+    int per = 1;
+    double least = 1e300;
+    for (int c = 1; c <= chunks; ++c) {  // the split whose busiest warp has the least to do
+        const long long n_items = (long long)n * ((chunks + c - 1) / c);
+        const double t = (double)((n_items + resident - 1) / resident) * (geometry + c);
+        if (t < least) {
+            least = t;
+            per = c;
+        }
+    }
     const long long items = (long long)n * ((chunks + per - 1) / per);
-    const long long blocks = std::min((items + kWarps - 1) / kWarps, (long long)152 * (JAC ? 8 : 16));
-    const size_t smem = offsets_smem<R>(pb) + (JAC ? sizeof(R) * kWarps * 32 * kNpar<FILL> : 0);
-    auto kern = k_models<R, NL, FILL, JAC>;
+    const long long blocks = std::min((items + kWarps - 1) / kWarps, (long long)resident / kWarps);
+    const size_t smem = offsets_smem<float>(pb) + (JAC ? sizeof(float) * kWarps * 32 * kNpar<FILL> : 0);
+    auto kern = k_models<NL, FILL, JAC>;
     cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<(int)blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, per, (R *)stokes, (R *)jac);
+    kern<<<(int)blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, per, (float *)stokes, (float *)jac);
     return cudaGetLastError();
 }
 
@@ -485,25 +544,29 @@ cudaError_t launch_synth(const KProblem &pb, int dtype, const double *params, co
     if (dtype != ME_F32)
         return pb.fill ? synth64_t<true>(pb, params, mu_px, n, stokes, st)
                        : synth64_t<false>(pb, params, mu_px, n, stokes, st);
-    if (pb.fill) return models_t<float, 0, true, false>(pb, params, mu_px, n, stokes, nullptr, st);
-    if (pb.n_lines == 1) return models_t<float, 1, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
-    if (pb.n_lines == 2) return models_t<float, 2, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
-    return models_t<float, 0, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    if (pb.fill) return models_t<0, true, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    if (pb.n_lines == 1) return models_t<1, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    if (pb.n_lines == 2) return models_t<2, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
+    return models_t<0, false, false>(pb, params, mu_px, n, stokes, nullptr, st);
 }
 
 cudaError_t launch_jac(const KProblem &pb, int dtype, const double *params, const double *mu_px,
                        int n, void *stokes, void *jac, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    if (pb.fill)
-        return dtype == ME_F32 ? models_t<float, 0, true, true>(pb, params, mu_px, n, stokes, jac, st)
-                               : models_t<double, 0, true, true>(pb, params, mu_px, n, stokes, jac, st);
-    if (dtype == ME_F32) {
-        if (pb.n_lines == 1) return models_t<float, 1, false, true>(pb, params, mu_px, n, stokes, jac, st);
-        if (pb.n_lines == 2) return models_t<float, 2, false, true>(pb, params, mu_px, n, stokes, jac, st);
-        return models_t<float, 0, false, true>(pb, params, mu_px, n, stokes, jac, st);
+    if (dtype != ME_F32) {
+        const int blocks = (int)(((long long)n * pb.n_lambda + kSynthBlock - 1) / kSynthBlock);
+        const size_t smem = offsets_smem<double>(pb);
+        if (pb.fill)
+            k_jac64<true><<<blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, (double *)stokes, (double *)jac);
+        else
+            k_jac64<false><<<blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, (double *)stokes, (double *)jac);
+        return cudaGetLastError();
     }
-    return models_t<double, 0, false, true>(pb, params, mu_px, n, stokes, jac, st);
+    if (pb.fill) return models_t<0, true, true>(pb, params, mu_px, n, stokes, jac, st);
+    if (pb.n_lines == 1) return models_t<1, false, true>(pb, params, mu_px, n, stokes, jac, st);
+    if (pb.n_lines == 2) return models_t<2, false, true>(pb, params, mu_px, n, stokes, jac, st);
+    return models_t<0, false, true>(pb, params, mu_px, n, stokes, jac, st);
 }
 
 cudaError_t launch_vjp(const KProblem &pb, int dtype, const double *params, const double *mu_px,
