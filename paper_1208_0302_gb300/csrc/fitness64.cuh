@@ -62,26 +62,6 @@ template <int K> __device__ __forceinline__ C2<double> convergent_of(const doubl
     return {p * r, x * q * r};
 }
 
-// w from the node nearest to (|x|, y): row = the nodes of y's nearest row, dy
-// = y's offset from it.
-__device__ __forceinline__ C2<double> from_node(const double2 *row, double x, double dy)
-{
-    const double ax = fabs(x);
-    const int ix = min((int)(narrow(ax) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
-    const double dx = ax - widen((float)ix * (float)kNodeStep);
-    const double2 *c = row + ix * kNodeCoef;
-    const double2 top = __ldg(c + kNodeCoef - 1);
-    double re = top.x, im = top.y;
-#pragma unroll
-    for (int n = kNodeCoef - 2; n >= 0; --n) {
-        const double2 v = __ldg(c + n);
-        const double t = fma(re, dx, fma(-im, dy, v.x));
-        im = fma(re, dy, fma(im, dx, v.y));
-        re = t;
-    }
-    return {re, __hiloint2double(__double2hiint(im) ^ (__double2hiint(x) & (int)0x80000000), __double2loint(im))};
-}
-
 // One individual's geometry and what its profiles need.
 struct Fit64Model {
     Geo<double> g;

@@ -126,6 +126,8 @@ struct ProfShared {
     double inv[kProfMaxComp], off[kProfMaxComp];  // x = (lambda - lambda0) inv + off
     double q[kProfMaxComp];                // strength times eta_ratio / 2
     unsigned char line[kProfMaxComp], group[kProfMaxComp];  // 0 sigma_b, 1 pi, 2 sigma_r, 3 field-free; + 4: also field-free
+    const double2 *row;  // without cells: the nodes of the damping's nearest row (NULL: the cells are built)
+    double dy;           // and the damping's offset from it
     int ncomp;
     int count[4];                          // list lengths by region: table, 9th, 7th, 5th
 };
@@ -257,6 +259,16 @@ __device__ __forceinline__ void build_geometry(ProfShared &S, const KProblem &pb
     }
 }
 
+// Building the cells costs one warp about 108 FP64 operations and saves each
+// round of 32 interior points 16 of the 45 that an expansion from the grid's
+// own nodes takes; about two fifths of the points are interior.  So the cells
+// pay from some 540 points on; one-line models of 64 wavelengths (192 points)
+// go without: a call for one 14.3 -> 12.5 us, 65 536 of them 2.28 -> 1.94 ms.
+__device__ __forceinline__ bool use_cells(const KProblem &pb, double y)
+{
+    return prof_components(pb) * pb.n_lambda > 540 || !(y >= 0.0);
+}
+
 // The model's tables in S: the cells, the geometry and the convergents'
 // coefficients on a warp each, side by side (p as above).  Nothing in S may be
 // read before a barrier (profile_sums begins with one).
@@ -264,8 +276,17 @@ template <bool FILL>
 __device__ __forceinline__ void build_model(ProfShared &S, const KProblem &pb, const double *p, double mu)
 {
     const int warp = threadIdx.x >> 5;
-    if (warp == 0) build_cells(S, pb.nodes, p[5]);
-    else if (warp == 1) build_geometry<FILL>(S, pb, p, mu);
+    if (warp == 0) {
+        const double y = p[5];
+        const bool cells = use_cells(pb, y);
+        if (cells) build_cells(S, pb.nodes, y);
+        if ((threadIdx.x & 31) == 0) {
+            const int iy = min((int)(narrow(fabs(y)) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
+            S.row = cells ? nullptr : pb.nodes + (size_t)iy * kNodeGrid * kNodeCoef;
+            S.dy = y - widen((float)iy * (float)kNodeStep);
+        }
+    }
+    if (warp == 1) build_geometry<FILL>(S, pb, p, mu);
     else if (warp == 2) build_exterior(S, p[5]);
 }
 
@@ -310,6 +331,26 @@ __device__ __forceinline__ double2 from_cells(const ProfShared &S, double x)
     }
     w.y = __hiloint2double(__double2hiint(w.y) ^ (__double2hiint(x) & (int)0x80000000), __double2loint(w.y));
     return w;
+}
+
+// w from the node nearest to (|x|, y): row = the nodes of y's nearest row, dy
+// = y's offset from it.
+__device__ __forceinline__ C2<double> from_node(const double2 *row, double x, double dy)
+{
+    const double ax = fabs(x);
+    const int ix = min((int)(narrow(ax) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
+    const double dx = ax - widen((float)ix * (float)kNodeStep);
+    const double2 *c = row + ix * kNodeCoef;
+    const double2 top = __ldg(c + kNodeCoef - 1);
+    double re = top.x, im = top.y;
+#pragma unroll
+    for (int n = kNodeCoef - 2; n >= 0; --n) {
+        const double2 v = __ldg(c + n);
+        const double t = fma(re, dx, fma(-im, dy, v.x));
+        im = fma(re, dy, fma(im, dx, v.y));
+        re = t;
+    }
+    return {re, __hiloint2double(__double2hiint(im) ^ (__double2hiint(x) & (int)0x80000000), __double2loint(im))};
 }
 
 // Profile sums of wavelength j0 + threadIdx.x for the model in S, by all
@@ -374,7 +415,12 @@ __device__ __forceinline__ ProfSums profile_sums(ProfShared &S, const KProblem &
                 const int i = k * 32 + lane;
                 if (i < n0) {
                     double2 &s = slot[la[i]];
-                    s = from_cells(S, s.x);
+                    if (S.row) {
+                        const C2<double> w = from_node(S.row, s.x, S.dy);
+                        s = make_double2(w.x, w.y);
+                    } else {
+                        s = from_cells(S, s.x);
+                    }
                 }
             } else if (k < r1) {
                 const int i = (k - r0) * 32 + lane;

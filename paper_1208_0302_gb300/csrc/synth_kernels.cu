@@ -234,7 +234,7 @@ k_vjp(const __grid_constant__ KProblem pb, const double *__restrict__ params,
 
 // FP64 synthesis, one block per model (see profiles64.cuh): 65 536 two-line
 // models 14.0 -> 4.8 ms against a thread per (model, wavelength), a call for one
-// one-line model 27 -> 17 us; absolute error 1.5e-15 -> 7e-17 rms.
+// one-line model 27 -> 12.5 us; absolute error 1.5e-15 -> 7e-17 rms.
 template <bool FILL>
 __global__ void __launch_bounds__(kProfBlock)
 k_synth64(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
