@@ -15,22 +15,22 @@ cudaError_t upload_tables_ga_fill(const HostTables &t)
 // Every line may carry a full pattern here (run-time check per line).
 cudaError_t launch_ga_evolve_fill(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
                                   const double *w, const double *mu_px, int npix, double *best,
-                                  uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub)
+                                  uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub, long long others)
 {
     if (npix <= 0) return cudaSuccess;
     constexpr int M = ME_NPAR_MAX;
     if (dtype == ME_F32) {
         if (ga.npop <= 256)
             return launch_evolve_t<float, 0, 256, false, true, M>(pb, ga, obs, w, mu_px, npix, best, best_genes,
-                                                                  st, nullptr, sd, sub);
+                                                                  st, nullptr, sd, sub, others);
         return launch_evolve_t<float, 0, 1024, false, true, M>(pb, ga, obs, w, mu_px, npix, best, best_genes,
-                                                               st, nullptr, sd, sub);
+                                                               st, nullptr, sd, sub, others);
     }
     if (ga.npop <= 256)
         return launch_evolve_t<double, 0, 256, false, true, M>(pb, ga, obs, w, mu_px, npix, best, best_genes,
-                                                               st, nullptr, sd, sub);
+                                                               st, nullptr, sd, sub, others);
     return launch_evolve_t<double, 0, 1024, false, true, M>(pb, ga, obs, w, mu_px, npix, best, best_genes,
-                                                            st, nullptr, sd, sub);
+                                                            st, nullptr, sd, sub, others);
 }
 
 }  // namespace genesis

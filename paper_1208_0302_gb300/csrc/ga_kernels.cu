@@ -101,13 +101,13 @@ bool has_pattern(const KProblem &pb)
 
 cudaError_t launch_ga_evolve(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
                              const double *w, const double *mu_px, int npix, double *best,
-                             uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub)
+                             uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub, long long others)
 {
     if (npix <= 0) return cudaSuccess;
-    if (pb.fill) return launch_ga_evolve_fill(pb, ga, dtype, obs, w, mu_px, npix, best, best_genes, st, sd, sub);
+    if (pb.fill) return launch_ga_evolve_fill(pb, ga, dtype, obs, w, mu_px, npix, best, best_genes, st, sd, sub, others);
     const bool pat = has_pattern(pb);
 #define GENESIS_EVOLVE(R, NL, MAXT, PAT) \
-    launch_evolve_t<R, NL, MAXT, false, PAT>(pb, ga, obs, w, mu_px, npix, best, best_genes, st, nullptr, sd, sub)
+    launch_evolve_t<R, NL, MAXT, false, PAT>(pb, ga, obs, w, mu_px, npix, best, best_genes, st, nullptr, sd, sub, others)
     if (dtype == ME_F32 && pat) {
         if (ga.npop <= 256) return GENESIS_EVOLVE(float, 0, 256, true);
         return GENESIS_EVOLVE(float, 0, 1024, true);

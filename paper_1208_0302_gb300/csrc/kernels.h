@@ -98,11 +98,12 @@ cudaError_t upload_nodes(void **ptr);
 // ga_kernels.cu
 cudaError_t launch_ga_evolve(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
                              const double *w, const double *mu_px, int npix, double *best,
-                             uint16_t *best_genes, cudaStream_t st, KSeed sd = {}, KSub sub = {});
+                             uint16_t *best_genes, cudaStream_t st, KSeed sd = {}, KSub sub = {},
+                             long long others = 0);  // warps that other launches fill meanwhile
 // ga_fill_kernels.cu: the same for problems with the fill fraction
 cudaError_t launch_ga_evolve_fill(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
                                   const double *w, const double *mu_px, int npix, double *best,
-                                  uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub);
+                                  uint16_t *best_genes, cudaStream_t st, KSeed sd, KSub sub, long long others);
 cudaError_t launch_ga_count(const KProblem &pb, const KGa &ga, int dtype, const void *obs,
                             const double *w, const double *mu_px, int npix, double *best,
                             unsigned long long *counts, cudaStream_t st);

@@ -132,8 +132,13 @@ int launch_request(serve_handle *h, Request *r)
     const double *dpw = r->pw.empty() ? dw : (const double *)(db + L.pw);
     double *dbest = (double *)(db + L.best);
     double *dchi2 = (double *)(db + L.chi2);
+    // the warps that the requests in flight and in the queue bring (the GA
+    // splits a small request while they leave the GPU room)
+    long long others = 0;
+    for (const Request *o : h->running) others += (long long)o->rq.npix * (o->rq.ga.npop / 32);
+    for (const Request *o : h->queue) others += (long long)o->rq.npix * (o->rq.ga.npop / 32);
     e = launch_ga_evolve(h->kp, g, h->pb.dtype, db + L.obs, q.ga.weight_mode == ME_W_USER ? dw : nullptr,
-                         dmu, q.npix, dbest, nullptr, st);
+                         dmu, q.npix, dbest, nullptr, st, {}, {}, others);
     if (e != cudaSuccess) return cuda_error(e, "serve GA launch");
     if (q.polish_iters > 0) {
         KLm lm;
