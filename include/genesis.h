@@ -429,7 +429,7 @@ int me_line_centre(const me_problem *pb, const void *obs, int npix, int half_wid
 
 /* ------------------------------------------ pixel selection and seeding
  * me_classify - Section 2 pixel selection with the weak-field fallback, and
- * the Section 5.5 seeds and polarity, one pixel per warp in FP64.
+ * the Section 5.5 seeds and polarity, in FP64.
  *   Threshold: I_c = mean of I over the quiet window [q_lo, q_hi); sigma_s^2
  *   the variance (1/n) of s = Q, U, V there; p = sqrt(Qmax^2 + Umax^2 +
  *   Vmax^2) / I_c with X_max = max |X| over the grid; sigma_P = p_thresh

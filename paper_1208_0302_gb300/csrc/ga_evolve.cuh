@@ -90,7 +90,9 @@ template <> struct GaDecode<double> {
     }
 };
 
-// Eq. chisq for one individual, FP32 (or FP64) synthesis over the whole grid.
+// Eq. chisq for one individual, synthesis over the whole grid: FP64 blocks of
+// more than 256 threads (smaller ones, whose convergents' coefficients fit
+// shared memory, take fitness64.cuh).
 // s_obs rows are (I, Q, U, V) of one wavelength; s_doff rows hold
 // lambda_j - lambda0_l for l = 0..3: one vector load each per wavelength.
 // STORE (verification kernel only): res, when not NULL, receives the
