@@ -1,6 +1,10 @@
 // Taylor coefficients of w(z) = exp(-z^2) erfc(-i z) at the nodes of a grid
-// over 0 <= x, y <= 10, computed on the host in double-double arithmetic so
-// that the rounded coefficients are correct to the last place or so.
+// over 0 <= x <= 10, -1.48 <= y <= 10, computed on the host in double-double
+// arithmetic so that the rounded coefficients are correct to the last place or
+// so.  (No physical damping lies below 0, but callers' own parameters and
+// per-pixel bounds may.  Weideman's series, which FP64 takes elsewhere, is 5e-7
+// from w at y = -1.5 and 4e-4 at -2, no better than the expansions of the last
+// row.)
 //
 // From w' = -2 z w + 2 i / sqrt(pi) the coefficients c_n = w^(n) / n! obey
 // c_{n+1} = -2 (z c_n + c_{n-1}) / (n + 1), n >= 1.  The first node is z = 10 i,
@@ -14,7 +18,8 @@
 
 namespace genesis {
 
-constexpr int kNodeGrid = 129;            // nodes per axis
+constexpr int kNodeGrid = 129;            // nodes per axis from 0 on
+constexpr int kNodeBelow = 19;            // rows below y = 0
 constexpr double kNodeStep = 0.078125;    // 10 / 128, exact
 constexpr int kNodeCoef = 11;             // coefficients kept per node
 
@@ -78,38 +83,69 @@ inline void taylor(double x, double y, CDD w, CDD c[kTerms])
 
 }  // namespace nodes
 
+namespace nodes {
+
+// w at the top node of the imaginary axis.
+inline CDD axis_top()
+{
+    const double y = (kNodeGrid - 1) * kNodeStep;
+    DD t = {y, 0.0};
+    for (int m = 300; m >= 1; --m) t = add({y, 0.0}, div({0.5 * m, 0.0}, t));
+    return {div({0x1.20dd750429b6dp-1, 0x1.1ae3a914fed80p-57}, t), {0.0, 0.0}};  // 1 / sqrt(pi) / t
+}
+
+// w at the axis node one row down from its expansion c: step -i h.
+inline CDD axis_down(const CDD c[kTerms])
+{
+    CDD w = c[kTerms - 1];
+    for (int n = kTerms - 2; n >= 0; --n)
+        w = {add(c[n].re, scale(w.im, kNodeStep)), add(c[n].im, scale(w.re, -kNodeStep))};
+    return w;
+}
+
+// The nodes of row iy from w on the axis, which moves one row down.
+inline void row(int iy, CDD &axis, double *o)
+{
+    CDD c[kTerms], w = axis;
+    for (int ix = 0; ix < kNodeGrid; ++ix, o += kNodeCoef * 2) {
+        taylor(ix * kNodeStep, iy * kNodeStep, w, c);
+        for (int n = 0; n < kNodeCoef; ++n) {
+            o[2 * n] = c[n].re.hi;
+            o[2 * n + 1] = c[n].im.hi;
+        }
+        if (ix == 0) axis = axis_down(c);
+        w = c[kTerms - 1];  // the next node of the row: step h
+        for (int n = kTerms - 2; n >= 0; --n)
+            w = {add(c[n].re, scale(w.re, kNodeStep)), add(c[n].im, scale(w.im, kNodeStep))};
+    }
+}
+
+}  // namespace nodes
+
+constexpr int kNodeRow = kNodeGrid * kNodeCoef * 2;  // doubles in a row of nodes
+
 // Row (iy, ix) holds (re, im) of c_0 .. c_10 at z = ix step + i iy step.  At
 // most half a step away on each axis the first omitted term is below 5e-17.
 inline std::vector<double> faddeeva_nodes()
 {
-    using namespace nodes;
-    std::vector<double> out((size_t)kNodeGrid * kNodeGrid * kNodeCoef * 2);
-    CDD c[kTerms], axis;
-    {
-        const double y = (kNodeGrid - 1) * kNodeStep;
-        DD t = {y, 0.0};
-        for (int m = 300; m >= 1; --m) t = add({y, 0.0}, div({0.5 * m, 0.0}, t));
-        axis = {div({0x1.20dd750429b6dp-1, 0x1.1ae3a914fed80p-57}, t), {0.0, 0.0}};  // 1 / sqrt(pi) / t
-    }
+    std::vector<double> out((size_t)kNodeGrid * kNodeRow);
+    nodes::CDD axis = nodes::axis_top();
+    for (int iy = kNodeGrid - 1; iy >= 0; --iy) nodes::row(iy, axis, &out[(size_t)iy * kNodeRow]);
+    return out;
+}
+
+// The kNodeBelow rows below, y = -kNodeBelow step first.  w grows like 2
+// exp(-z^2) there, and so does an error, so the relative accuracy stays; the
+// expansions stay within 1e-13 |w|, 1e-14 down to y = -1.
+inline std::vector<double> faddeeva_nodes_below()
+{
+    std::vector<double> out((size_t)kNodeBelow * kNodeRow);
+    nodes::CDD axis = nodes::axis_top(), c[nodes::kTerms];
     for (int iy = kNodeGrid - 1; iy >= 0; --iy) {
-        CDD w = axis;
-        for (int ix = 0; ix < kNodeGrid; ++ix) {
-            taylor(ix * kNodeStep, iy * kNodeStep, w, c);
-            double *o = &out[((size_t)iy * kNodeGrid + ix) * kNodeCoef * 2];
-            for (int n = 0; n < kNodeCoef; ++n) {
-                o[2 * n] = c[n].re.hi;
-                o[2 * n + 1] = c[n].im.hi;
-            }
-            if (ix == 0 && iy > 0) {  // the axis node one row down: step -i h
-                axis = c[kTerms - 1];
-                for (int n = kTerms - 2; n >= 0; --n)
-                    axis = {add(c[n].re, scale(axis.im, kNodeStep)), add(c[n].im, scale(axis.re, -kNodeStep))};
-            }
-            w = c[kTerms - 1];  // the next node of the row: step h
-            for (int n = kTerms - 2; n >= 0; --n)
-                w = {add(c[n].re, scale(w.re, kNodeStep)), add(c[n].im, scale(w.im, kNodeStep))};
-        }
+        nodes::taylor(0.0, iy * kNodeStep, axis, c);
+        axis = nodes::axis_down(c);
     }
+    for (int iy = -1; iy >= -kNodeBelow; --iy) nodes::row(iy, axis, &out[(size_t)(iy + kNodeBelow) * kNodeRow]);
     return out;
 }
 

@@ -73,9 +73,7 @@ __device__ __forceinline__ Fit64Model fit64_model(const KProblem &pb, const doub
 {
     Fit64Model m;
     m.g = make_geo<double, 0, FILL>(pb, pb.n_lines, p, mu);
-    const int iy = min((int)(narrow(m.g.a) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
-    m.row = pb.nodes + (size_t)iy * kNodeGrid * kNodeCoef;
-    m.dy = m.g.a - widen((float)iy * (float)kNodeStep);
+    m.row = node_row(pb.nodes, m.g.a, m.dy);
     return m;
 }
 

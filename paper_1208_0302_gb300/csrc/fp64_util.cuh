@@ -16,8 +16,9 @@ __device__ __forceinline__ double widen(float x)
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// x >= 0 truncated to FP32 with integer operations; 0 below FP32's normal
-// range, the largest finite value above it (and for NaN).
+// x >= 0, sign bit clear (a set one, -0 included, reads as a huge value),
+// truncated to FP32 with integer operations; 0 below FP32's normal range, the
+// largest finite value above it (and for NaN).
 __device__ __forceinline__ float narrow(double x)
 {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);

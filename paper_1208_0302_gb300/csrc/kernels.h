@@ -92,7 +92,7 @@ cudaError_t upload_tables_lm(const HostTables &t);
 cudaError_t upload_tables_ga_fill(const HostTables &t);
 cudaError_t upload_tables_check(const HostTables &t);
 // The file-scope array of w's Taylor coefficients (synth_kernels.cu), filled on
-// the current device; *ptr receives its address (KProblem::nodes).
+// the current device; *ptr receives the address of row y = 0 (KProblem::nodes).
 cudaError_t upload_nodes(void **ptr);
 
 // ga_kernels.cu

@@ -56,7 +56,7 @@ struct KProblem {
     double mu;
     KLine line[ME_MAX_LINES];
     double lam[ME_MAX_LAMBDA];  // wavelength grid [A]
-    const double2 *nodes;       // device: FP64 Taylor coefficients of w (faddeeva_nodes.h)
+    const double2 *nodes;       // device: FP64 Taylor coefficients of w (faddeeva_nodes.h), at row y = 0
 };
 
 // Weideman coefficient tables (filled per device at library initialisation).

@@ -147,16 +147,26 @@ inline size_t prof_smem(const KProblem &pb)
     return sizeof(ProfShared) + (size_t)c * kProfBlock * (sizeof(double2) + 2 * sizeof(unsigned short));
 }
 
+// The row of nodes nearest to damping y and y's offset from it.  Dampings
+// beyond the grid's ends get its first or last row.
+__device__ __forceinline__ const double2 *node_row(const double2 *nodes, double y, double &dy)
+{
+    const double t = y + kNodeBelow * kNodeStep;  // also takes -0, whose bits are not those of 0
+    const int n = __double2hiint(t) < 0 ? 0 : (int)(narrow(t) * (float)(1.0 / kNodeStep) + 0.5f);
+    const int iy = min(n, kNodeBelow + kNodeGrid - 1) - kNodeBelow;
+    dy = y - widen((float)iy * (float)kNodeStep);
+    return nodes + iy * (kNodeGrid * kNodeCoef);
+}
+
 // One warp: the Taylor table of damping y, a cell per lane.
 __device__ __forceinline__ void build_cells(ProfShared &S, const double2 *nodes, double y)
 {
     const int lane = threadIdx.x & 31;
     const double x = (lane + 0.5) * kCellWidth;
     C2<double> m;
-    if (y >= 0.0) {  // from the node at x and the nearest y: a step along i
-        const int iy = min((int)(narrow(y) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
-        const double2 *c = nodes + ((size_t)iy * kNodeGrid + 4 * lane + 2) * kNodeCoef;
-        const double dy = y - widen((float)iy * (float)kNodeStep);
+    if (y >= -kNodeBelow * kNodeStep) {  // from the node at x and the nearest y: a step along i
+        double dy;
+        const double2 *c = node_row(nodes, y, dy) + (4 * lane + 2) * kNodeCoef;
         const double2 top = __ldg(c + kNodeCoef - 1);
         m = {top.x, top.y};
 #pragma unroll
@@ -266,7 +276,7 @@ __device__ __forceinline__ void build_geometry(ProfShared &S, const KProblem &pb
 // go without: a call for one 14.3 -> 12.5 us, 65 536 of them 2.28 -> 1.94 ms.
 __device__ __forceinline__ bool use_cells(const KProblem &pb, double y)
 {
-    return prof_components(pb) * pb.n_lambda > 540 || !(y >= 0.0);
+    return prof_components(pb) * pb.n_lambda > 540 || !(y >= -kNodeBelow * kNodeStep);
 }
 
 // The model's tables in S: the cells, the geometry and the convergents'
@@ -281,9 +291,10 @@ __device__ __forceinline__ void build_model(ProfShared &S, const KProblem &pb, c
         const bool cells = use_cells(pb, y);
         if (cells) build_cells(S, pb.nodes, y);
         if ((threadIdx.x & 31) == 0) {
-            const int iy = min((int)(narrow(fabs(y)) * (float)(1.0 / kNodeStep) + 0.5f), kNodeGrid - 1);
-            S.row = cells ? nullptr : pb.nodes + (size_t)iy * kNodeGrid * kNodeCoef;
-            S.dy = y - widen((float)iy * (float)kNodeStep);
+            double dy;
+            const double2 *row = node_row(pb.nodes, y, dy);
+            S.row = cells ? nullptr : row;
+            S.dy = dy;
         }
     }
     if (warp == 1) build_geometry<FILL>(S, pb, p, mu);

@@ -10,13 +10,17 @@
 
 namespace genesis {
 
-static __device__ double2 d_nodes[kNodeGrid * kNodeGrid * kNodeCoef];
+static __device__ double2 d_nodes[(kNodeBelow + kNodeGrid) * kNodeGrid * kNodeCoef];
 
 cudaError_t upload_nodes(void **ptr)
 {
-    static const std::vector<double> host = faddeeva_nodes();
-    const cudaError_t e = cudaGetSymbolAddress(ptr, d_nodes);
-    return e != cudaSuccess ? e : cudaMemcpyToSymbol(d_nodes, host.data(), sizeof(d_nodes));
+    static const std::vector<double> below = faddeeva_nodes_below(), host = faddeeva_nodes();
+    const size_t nb = below.size() * sizeof(double);
+    cudaError_t e = cudaGetSymbolAddress(ptr, d_nodes);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(d_nodes, below.data(), nb);
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(d_nodes, host.data(), host.size() * sizeof(double), nb);
+    *ptr = (char *)*ptr + nb;  // row 0
+    return e;
 }
 
 cudaError_t upload_tables_synth(const HostTables &t)
