@@ -9,13 +9,17 @@
 
 namespace genesis {
 
-// Let a kernel take `bytes` of dynamic shared memory.  A call to the runtime
-// is needed only above the 48 KB that every kernel may have, static arrays (at
-// most 8 KB here) included.
+// Let a kernel take `bytes` of dynamic shared memory.  The limit belongs to the
+// kernel, not to the launch, and host threads share it: every call that has to
+// raise it sets the same value, what a block can have on sm_103a (227 KB) less
+// the static arrays beside it (3 KB, more than any kernel here declares), so
+// no thread lowers it between another's call and launch.  Up to 40 KB needs no
+// call to the runtime: every kernel may have 48 KB in all.
+constexpr size_t kMaxDynamicSmem = 224 * 1024;
 template <class Kernel> inline cudaError_t allow_smem(Kernel kern, size_t bytes)
 {
     if (bytes <= 40 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynamicSmem);
 }
 
 // GA launch parameters (Section 3 operators, Section 5.6 restarts).
