@@ -25,12 +25,9 @@ ALL_FREE = (1 << NPAR_MAX) - 1
 # pointers and one pass of checks an autograd step of a small batch went from
 # 215 to 190 us (105 of them an empty autograd function) and me_synth from 20
 # to 11 us of host time.
-_raw_stream = torch._C._cuda_getCurrentRawStream
-_device = torch._C._cuda_getDevice
-
-
 def _stream():
-    return _raw_stream(_device())
+    # looked up here: a PyTorch without CUDA does not have them
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
