@@ -98,50 +98,8 @@ __device__ __forceinline__ double fit64_share(const KProblem &pb, int nl, const 
 {
     double sum = 0.0, comp = 0.0;
     for (int j = r; j < nl; j += kShares) {
-        ProfSums S = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll 1
-        for (int l = 0; l < pb.n_lines; ++l) {
-            const KLine &ln = pb.line[l];
-            const double x0 = fma(s_doff[4 * j + l], m.g.invD[l], m.g.cp[l]);
-            const double q = ln.half_eta;
-            if (ln.ncomp[0] == 0) {
-#pragma unroll 1
-                for (int c = 0; c < 3; ++c) {
-                    const double x = c == 0 ? x0 + m.g.vB[l] : c == 1 ? x0 : x0 - m.g.vB[l];
-                    const C2<double> w = fit64_profile(m, coef, n, x);
-                    if (c == 0) {
-                        S.Sb = fma(q, w.x, S.Sb);
-                        S.Sbi = fma(q, w.y, S.Sbi);
-                    } else if (c == 1) {
-                        S.P = fma(q, w.x, S.P);
-                        S.Pi = fma(q, w.y, S.Pi);
-                        if (FILL) S.P0 = fma(q, w.x, S.P0);
-                    } else {
-                        S.Sr = fma(q, w.x, S.Sr);
-                        S.Sri = fma(q, w.y, S.Sri);
-                    }
-                }
-            } else {
-#pragma unroll 1
-                for (int g = 0; g < 3; ++g)
-#pragma unroll 1
-                    for (int i = 0; i < ln.ncomp[g]; ++i) {
-                        const C2<double> w = fit64_profile(m, coef, n, fma(-m.g.vL[l], ln.cshift[g][i], x0));
-                        const double qc = q * ln.cstr[g][i];
-                        if (g == 0) {
-                            S.Sb = fma(qc, w.x, S.Sb);
-                            S.Sbi = fma(qc, w.y, S.Sbi);
-                        } else if (g == 1) {
-                            S.P = fma(qc, w.x, S.P);
-                            S.Pi = fma(qc, w.y, S.Pi);
-                        } else {
-                            S.Sr = fma(qc, w.x, S.Sr);
-                            S.Sri = fma(qc, w.y, S.Sri);
-                        }
-                    }
-                if (FILL) S.P0 = fma(q, fit64_profile(m, coef, n, x0).x, S.P0);
-            }
-        }
+        const ProfSums S = point_sums<FILL>(pb, m.g, [&](int l) { return s_doff[4 * j + l]; },
+                                            [&](double x) { return fit64_profile(m, coef, n, x); });
         const Stokes4<double> s = stokes_of<FILL>(m.g, S);
         const double r0 = s_obs[4 * j] - s.I, r1 = s_obs[4 * j + 1] - s.Q, r2 = s_obs[4 * j + 2] - s.U,
                      r3 = s_obs[4 * j + 3] - s.V;

@@ -1,0 +1,63 @@
+// Launch shapes by sizes: which of a call's kernels runs, and how its work is
+// dealt out.  Plain C++ without CUDA, so that the rules can be tested on any
+// host.  The constants are fits to times measured on a GB300; each rule says
+// over which sizes.
+#pragma once
+
+#include <algorithm>
+
+namespace genesis {
+
+constexpr int kSMs = 152;  // of a whole GB300
+
+// FP32 synthesis and Jacobian: how many chunks of 32 wavelengths of one model
+// a warp takes (k_models), or 0 for a thread per (model, wavelength)
+// (k_points).  k_models forms a model's geometry once per warp and not once
+// per lane, but a chunk's lanes beyond the grid idle and equal shares of the
+// models' unequal work are dealt to the warps beforehand; k_points leaves no
+// lane idle and its blocks are dealt out as they finish.
+//  * Fewer than one and a half rounds of resident warps: k_models, which is
+//    the faster or within 15 % there, but for heavy models.
+//  * Heavy models (more than 40 Zeeman components): k_points below 448
+//    wavelengths (69 components, 30 000 models: 64 wavelengths 473 -> 386 us,
+//    129 869 -> 638, 384 level, 512 2314 against 2618).
+//  * Otherwise the smaller of the costs of a model: a fit to 1100 times of 600
+//    to 30 000 models of 3 to 512 wavelengths and 3 to 15 components, which
+//    picks the slower kernel by more than 6 % in 6 of them.  30 000 models,
+//    k_models against k_points: two lines, 8 wavelengths 35 -> 13 us, 33
+//    wavelengths 46 -> 37, 64 45.7 against 54; full pattern and a line, 33
+//    wavelengths 93 -> 62, 97 168 -> 139, 192 233 against 259; Jacobians of
+//    two lines, 8 wavelengths 62 -> 43, 33 99 against 117.
+// ncomp: Zeeman components of all lines; triplets: one or two effective triplets
+// without the fill fraction; blocks_per_sm: k_models's.
+inline int chunks_per_warp(bool jac, int n, int nl, int n_lines, int ncomp, bool triplets, int blocks_per_sm)
+{
+    const int resident = kSMs * blocks_per_sm * 4;  // warps of k_models on the chip
+    const int chunks = (nl + 31) / 32;
+    if (ncomp > 40) {
+        if (nl < 448) return 0;
+    } else if ((long long)n * chunks * 2 >= 3ll * resident) {
+        // per warp: k_points' and k_models' geometry, the closed form, a component
+        const double point_geo = jac ? (triplets ? 0.30 : 0.186 * n_lines) : triplets ? 0.052 : 0.0276 * n_lines;
+        const double model_geo = jac ? (triplets ? 0.02 : 0.063 * n_lines) : triplets ? 0.032 : 0.021 * n_lines;
+        const double closed = jac ? (triplets ? 0.125 : 0.055) : triplets ? 0.012 : 0.0;
+        const double comp = jac ? (triplets ? 0.0145 : 0.0212) : triplets ? 0.0092 : 0.0133;
+        const double chunk = closed + comp * ncomp;
+        if (nl / 32.0 * (point_geo + chunk) < model_geo + chunks * chunk) return 0;
+    }
+    // the split whose busiest warp has the least to do, the geometry counted in chunks
+    const double geometry = jac ? 0.2 : 0.8;
+    int per = 1;
+    double least = 1e300;
+    for (int c = 1; c <= chunks; ++c) {
+        const long long items = (long long)n * ((chunks + c - 1) / c);
+        const double t = (double)((items + resident - 1) / resident) * (geometry + c);
+        if (t < least) {
+            least = t;
+            per = c;
+        }
+    }
+    return per;
+}
+
+}  // namespace genesis

@@ -364,6 +364,67 @@ __device__ __forceinline__ C2<double> from_node(const double2 *row, double x, do
     return {re, __hiloint2double(__double2hiint(im) ^ (__double2hiint(x) & (int)0x80000000), __double2loint(im))};
 }
 
+// Profile sums of one wavelength by one thread: doff(l) = lambda - lambda0_l,
+// profile(x) = w(x + i a) for the model of geometry g.
+template <bool FILL, class Offset, class Profile>
+__device__ __forceinline__ ProfSums point_sums(const KProblem &pb, const Geo<double> &g, Offset doff, Profile profile)
+{
+    ProfSums S = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+    for (int l = 0; l < pb.n_lines; ++l) {
+        const KLine &ln = pb.line[l];
+        const double x0 = fma(doff(l), g.invD[l], g.cp[l]);
+        const double q = ln.half_eta;
+        if (ln.ncomp[0] == 0) {
+#pragma unroll 1
+            for (int c = 0; c < 3; ++c) {
+                const double x = c == 0 ? x0 + g.vB[l] : c == 1 ? x0 : x0 - g.vB[l];
+                const C2<double> w = profile(x);
+                if (c == 0) {
+                    S.Sb = fma(q, w.x, S.Sb);
+                    S.Sbi = fma(q, w.y, S.Sbi);
+                } else if (c == 1) {
+                    S.P = fma(q, w.x, S.P);
+                    S.Pi = fma(q, w.y, S.Pi);
+                    if (FILL) S.P0 = fma(q, w.x, S.P0);
+                } else {
+                    S.Sr = fma(q, w.x, S.Sr);
+                    S.Sri = fma(q, w.y, S.Sri);
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int k = 0; k < 3; ++k)
+#pragma unroll 1
+                for (int i = 0; i < ln.ncomp[k]; ++i) {
+                    const C2<double> w = profile(fma(-g.vL[l], ln.cshift[k][i], x0));
+                    const double qc = q * ln.cstr[k][i];
+                    if (k == 0) {
+                        S.Sb = fma(qc, w.x, S.Sb);
+                        S.Sbi = fma(qc, w.y, S.Sbi);
+                    } else if (k == 1) {
+                        S.P = fma(qc, w.x, S.P);
+                        S.Pi = fma(qc, w.y, S.Pi);
+                    } else {
+                        S.Sr = fma(qc, w.x, S.Sr);
+                        S.Sri = fma(qc, w.y, S.Sri);
+                    }
+                }
+            if (FILL) S.P0 = fma(q, profile(x0).x, S.P0);
+        }
+    }
+    return S;
+}
+
+// w(x + i a) for a thread on its own: the nearest node's expansion for |z|^2 <
+// 100 and the 9th convergent in complex arithmetic beyond (row and dy as in
+// from_node).
+__device__ __forceinline__ C2<double> profile_alone(const double2 *row, double dy, double x, double a, double a2)
+{
+    if (__double_as_longlong(fma(x, x, a2)) < 0x4059000000000000ll) return from_node(row, x, dy);  // 100, as bits
+    return faddeeva_exterior<double>(x, a, a2);
+}
+
 // Profile sums of wavelength j0 + threadIdx.x for the model in S, by all
 // kProfBlock threads (those beyond nl help and get zeros).  Every thread of
 // the block calls it (barriers inside, the first before anything in S is

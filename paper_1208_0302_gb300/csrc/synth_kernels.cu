@@ -4,6 +4,7 @@
 
 #include "async_copy.cuh"
 #include "kernels.h"
+#include "launch_rules.h"
 #include "me_jac.cuh"
 #include "profiles64.cuh"
 #include "rng_device.cuh"
@@ -138,50 +139,64 @@ k_models(const __grid_constant__ KProblem pb, const double *__restrict__ params,
     }
 }
 
-// FP64 Jacobian, one thread per (model, wavelength): bound by the FP64 pipe,
-// where the warp-per-model form above was 0 to 5 % slower (700 full-pattern
-// models 556 against 525 us).
-template <bool FILL>
+// Synthesis, and with JAC the Jacobian, a thread per (model, wavelength): every
+// lane works whatever the grid, but each forms its model's geometry.  FP32: see
+// chunks_per_warp.  The FP64 Jacobian always runs here: it is bound by the FP64
+// pipe, where a warp per model was 0 to 5 % slower (700 full-pattern models 556
+// against 525 us).
+template <class R, int NL, bool FILL, bool JAC>
 __global__ void __launch_bounds__(kSynthBlock)
-k_jac64(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px, int n,
-        double *__restrict__ stokes, double *__restrict__ jac)
+k_points(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px, int n,
+         R *__restrict__ stokes, R *__restrict__ jac)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int nl = pb.n_lambda, nlines = pb.n_lines;
-    double *s_he = (double *)smem;
-    double *s_doff = s_he + ME_MAX_LINES;
-    stage_offsets<double>(pb, nlines, s_doff, s_he);
+    const int nl = pb.n_lambda, nlines = NL > 0 ? NL : pb.n_lines;
+    R *s_he = (R *)smem;
+    R *s_doff = s_he + ME_MAX_LINES;
+    stage_offsets<R>(pb, nlines, s_doff, s_he);
     __syncthreads();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)n * nl) return;
     const int m = (int)(i / nl), j = (int)(i - (long long)m * nl);
     constexpr int M = kNpar<FILL>;
-    double p[M];
+    R p[M];
 #pragma unroll
-    for (int d = 0; d < M; ++d) p[d] = params[(size_t)m * M + d];
-    const double mu = mu_px ? mu_px[m] : pb.mu;
-    const GeoJ<double> G = make_geoj<double, 0, FILL>(pb, nlines, p, mu);
-    double doff[ME_MAX_LINES], he[ME_MAX_LINES];
+    for (int d = 0; d < M; ++d) p[d] = R(params[(size_t)m * M + d]);
+    const R mu = mu_px ? R(mu_px[m]) : R(pb.mu);
+    std::conditional_t<JAC, GeoJ<R>, Geo<R>> G;
+    if constexpr (JAC) G = make_geoj<R, NL, FILL>(pb, nlines, p, mu);
+    else G = make_geo<R, NL, FILL>(pb, nlines, p, mu);
+    Stokes4<R> s;
+    R J[4][M];
+    if constexpr (!JAC && sizeof(R) == 8) {
+        double dy;
+        const double2 *row = node_row(pb.nodes, G.a, dy);
+        s = stokes_of<FILL>(G, point_sums<FILL>(pb, G, [&](int l) { return s_doff[l * nl + j]; },
+                                                [&](double x) { return profile_alone(row, dy, x, G.a, G.a2); }));
+    } else {
+        R doff[ME_MAX_LINES], he[ME_MAX_LINES];
 #pragma unroll
-    for (int l = 0; l < ME_MAX_LINES; ++l) {
-        doff[l] = l < nlines ? s_doff[l * nl + j] : 0.0;
-        he[l] = s_he[l];
+        for (int l = 0; l < ME_MAX_LINES; ++l) {
+            doff[l] = l < nlines ? s_doff[l * nl + j] : R(0);
+            he[l] = s_he[l];
+        }
+        if constexpr (JAC) me_point_jac<R, NL, FILL>(G, doff, he, nlines, pb.line, s, J);
+        else s = me_point<R, NL, true, FILL>(G, doff, he, nlines, pb.line);
     }
-    Stokes4<double> s;
-    double J[4][M];
-    me_point_jac<double, 0, FILL>(G, doff, he, nlines, pb.line, s, J);
     if (stokes) {
-        double *o = stokes + (size_t)m * 4 * nl;
+        R *o = stokes + (size_t)m * 4 * nl;
         o[j] = s.I;
         o[nl + j] = s.Q;
         o[2 * nl + j] = s.U;
         o[3 * nl + j] = s.V;
     }
+    if constexpr (JAC) {
 #pragma unroll
-    for (int st = 0; st < 4; ++st) {
-        double *o = jac + (((size_t)m * 4 + st) * nl + j) * M;
+        for (int st = 0; st < 4; ++st) {
+            R *o = jac + (((size_t)m * 4 + st) * nl + j) * M;
 #pragma unroll
-        for (int k = 0; k < M; ++k) o[k] = J[st][k];
+            for (int k = 0; k < M; ++k) o[k] = J[st][k];
+        }
     }
 }
 
@@ -253,7 +268,7 @@ k_synth64(const __grid_constant__ KProblem pb, const double *__restrict__ params
     for (int d = 0; d < M; ++d) p[d] = params[(size_t)m * M + d];
     build_model<FILL>(S, pb, p, mu_px ? mu_px[m] : pb.mu);
     double *o = stokes + (size_t)m * 4 * nl;
-    for (int j0 = 0; j0 < nl; j0 += kProfBlock) {
+    for (int j0 = blockIdx.y * kProfBlock; j0 < nl; j0 += gridDim.y * kProfBlock) {
         const ProfSums r = profile_sums<FILL>(S, pb, j0, nl);
         const int j = j0 + threadIdx.x;
         if (j < nl) {
@@ -488,27 +503,28 @@ template <class R> size_t offsets_smem(const KProblem &pb)
     return sizeof(R) * (ME_MAX_LINES + (size_t)pb.n_lines * pb.n_lambda);
 }
 
+template <class R, int NL, bool FILL, bool JAC>
+cudaError_t points_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes, void *jac,
+                     cudaStream_t st)
+{
+    const long long blocks = ((long long)n * pb.n_lambda + kSynthBlock - 1) / kSynthBlock;
+    k_points<R, NL, FILL, JAC><<<(int)blocks, kSynthBlock, offsets_smem<R>(pb), st>>>(pb, params, mu_px, n, (R *)stokes,
+                                                                                    (R *)jac);
+    return cudaGetLastError();
+}
+
 template <int NL, bool FILL, bool JAC>
 cudaError_t models_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes, void *jac,
                      cudaStream_t st)
 {
     constexpr int kWarps = kSynthBlock / 32;
-    // resident warps, and a model's geometry in units of a chunk's work
-    const int resident = 152 * (JAC ? kJacMinB : 8) * kWarps;
-    const double geometry = JAC ? 0.2 : 0.8;
+    constexpr int kBlocks = JAC ? kJacMinB : 8;  // resident per SM
     const int chunks = (pb.n_lambda + 31) / 32;
-    int per = 1;
-    double least = 1e300;
-    for (int c = 1; c <= chunks; ++c) {  // the split whose busiest warp has the least to do
-        const long long n_items = (long long)n * ((chunks + c - 1) / c);
-        const double t = (double)((n_items + resident - 1) / resident) * (geometry + c);
-        if (t < least) {
-            least = t;
-            per = c;
-        }
-    }
+    const int per = chunks_per_warp(JAC, n, pb.n_lambda, pb.n_lines, prof_components(pb), NL > 0 && !has_pattern(pb),
+                                    kBlocks);
+    if (per == 0) return points_t<float, NL, FILL, JAC>(pb, params, mu_px, n, stokes, jac, st);
     const long long items = (long long)n * ((chunks + per - 1) / per);
-    const long long blocks = std::min((items + kWarps - 1) / kWarps, (long long)resident / kWarps);
+    const long long blocks = std::min((items + kWarps - 1) / kWarps, (long long)kSMs * kBlocks);
     const size_t smem = offsets_smem<float>(pb) + (JAC ? sizeof(float) * kWarps * 32 * kNpar<FILL> : 0);
     auto kern = k_models<NL, FILL, JAC>;
     cudaError_t e = allow_smem(kern, smem);
@@ -558,15 +574,9 @@ cudaError_t launch_jac(const KProblem &pb, int dtype, const double *params, cons
                        int n, void *stokes, void *jac, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    if (dtype != ME_F32) {
-        const int blocks = (int)(((long long)n * pb.n_lambda + kSynthBlock - 1) / kSynthBlock);
-        const size_t smem = offsets_smem<double>(pb);
-        if (pb.fill)
-            k_jac64<true><<<blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, (double *)stokes, (double *)jac);
-        else
-            k_jac64<false><<<blocks, kSynthBlock, smem, st>>>(pb, params, mu_px, n, (double *)stokes, (double *)jac);
-        return cudaGetLastError();
-    }
+    if (dtype != ME_F32)
+        return pb.fill ? points_t<double, 0, true, true>(pb, params, mu_px, n, stokes, jac, st)
+                       : points_t<double, 0, false, true>(pb, params, mu_px, n, stokes, jac, st);
     if (pb.fill) return models_t<0, true, true>(pb, params, mu_px, n, stokes, jac, st);
     if (pb.n_lines == 1) return models_t<1, false, true>(pb, params, mu_px, n, stokes, jac, st);
     if (pb.n_lines == 2) return models_t<2, false, true>(pb, params, mu_px, n, stokes, jac, st);

@@ -1,0 +1,62 @@
+"""The launch rules by sizes (csrc/launch_rules.h) against times measured on a
+GB300: where one of two kernels took at least 1.2 times the other's time, the
+rule has to pick the faster."""
+import os
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1208_0302_gb300", "csrc")
+MAIN = r"""
+#include <cstdio>
+#include <cstring>
+#include "launch_rules.h"
+using namespace genesis;
+int main()
+{
+    char rule[32];
+    while (std::scanf("%31s", rule) == 1) {
+        if (!std::strcmp(rule, "models")) {
+            int jac, lines, ncomp, triplets, nl, n;
+            if (std::scanf("%d %d %d %d %d %d", &jac, &lines, &ncomp, &triplets, &nl, &n) != 6) return 1;
+            std::printf("%d\n", chunks_per_warp(jac, n, nl, lines, ncomp, triplets, jac ? 4 : 8));
+        }
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    src = d / "rules.cpp"
+    src.write_text(MAIN)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-Wall", "-Werror", "-I", CSRC, "-o", str(d / "rules"), str(src)], check=True)
+
+    def run(calls):
+        text = "\n".join(" ".join(str(x) for x in c) for c in calls)
+        out = subprocess.run([str(d / "rules")], input=text, capture_output=True, text=True, check=True).stdout
+        return [[float(x) for x in line.split()] for line in out.splitlines()]
+
+    return run
+
+
+# (Jacobian, lines, components, triplets, wavelengths, models): us of k_points, us of k_models
+MODELS = [((1, 1, 3, 1, 8, 30000), 38.7, 47.6), ((1, 1, 3, 1, 24, 8000), 32.8, 16.5), ((1, 1, 3, 1, 65, 8000), 59.9, 35.3),
+          ((1, 1, 3, 1, 256, 600), 25.3, 14.9), ((1, 1, 3, 1, 257, 2500), 64.9, 33.3), ((1, 2, 6, 1, 8, 30000), 42.7, 62.3),
+          ((1, 2, 6, 1, 20, 30000), 77.0, 62.9), ((1, 2, 6, 1, 128, 8000), 103.9, 56.1),
+          ((1, 2, 6, 1, 129, 30000), 380.9, 223.9), ((1, 2, 15, 0, 6, 8000), 17.0, 30.4), ((1, 2, 15, 0, 32, 8000), 43.8, 31.2),
+          ((1, 2, 15, 0, 32, 30000), 123.8, 102.2), ((1, 2, 15, 0, 257, 30000), 808.7, 616.3),
+          ((1, 3, 9, 0, 65, 8000), 88.7, 66.0), ((1, 3, 9, 0, 192, 8000), 223.7, 127.2),
+          ((1, 4, 69, 0, 16, 30000), 172.6, 378.3), ((1, 4, 69, 0, 64, 8000), 164.9, 205.0),
+          ((1, 4, 69, 0, 128, 2500), 106.3, 128.9), ((0, 1, 3, 1, 97, 30000), 68.1, 51.8), ((0, 2, 6, 1, 8, 30000), 12.8, 35.2),
+          ((0, 2, 6, 1, 96, 30000), 87.1, 68.2), ((0, 2, 6, 1, 129, 8000), 37.4, 29.6), ((0, 2, 6, 1, 512, 30000), 1025.7, 211.7),
+          ((0, 2, 15, 0, 20, 30000), 39.4, 68.5), ((0, 2, 15, 0, 33, 30000), 62.4, 93.1), ((0, 2, 15, 0, 512, 8000), 295.4, 154.3),
+          ((0, 3, 9, 0, 192, 30000), 288.2, 153.1), ((0, 4, 69, 0, 12, 2500), 19.0, 32.7), ((0, 4, 69, 0, 32, 30000), 220.1, 271.0),
+          ((0, 4, 69, 0, 48, 8000), 90.9, 122.1)]
+
+
+def test_models_or_points(rule):
+    for (case, points, models), (per,) in zip(MODELS, rule([("models",) + m[0] for m in MODELS])):
+        assert (per == 0) == (points < models), (case, per)
+        assert per <= (case[4] + 31) // 32
