@@ -25,9 +25,13 @@ ALL_FREE = (1 << NPAR_MAX) - 1
 # pointers and one pass of checks an autograd step of a small batch went from
 # 215 to 190 us (105 of them an empty autograd function) and me_synth from 20
 # to 11 us of host time.
+# (None in a PyTorch without CUDA, where no tensor gets as far as a stream.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    # looked up here: a PyTorch without CUDA does not have them
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return _raw_stream(_device())
 
 
 def _ptr(t):
