@@ -60,4 +60,24 @@ inline int chunks_per_warp(bool jac, int n, int nl, int n_lines, int ncomp, bool
     return per;
 }
 
+// FP64 synthesis: blocks per model (k_synth64, whose passes of 128 wavelengths
+// they share), or 0 for a thread per (model, wavelength) (k_points).
+//  * A block works for one model, so on a few wavelengths most of its time goes
+//    into the model's tables; from 2000 models of up to 12 wavelengths on (6
+//    with more than 40 components) threads of their own are faster: 20 000
+//    models, one line, 3 wavelengths 326 -> 66 us, 8 339 -> 143, 16 362 -> 269;
+//    two lines, 12 wavelengths 434 -> 352, 16 462 against 460; four full
+//    patterns, 6 wavelengths 2802 -> 1797, 12 3257 against 3309.  Below 2000
+//    models a block each is faster (600 models of 8 wavelengths 16.5 against
+//    20.9 us).
+//  * Up to 152 models each get a block per pass, so that the passes run side by
+//    side: a call for one model, one line, 257 wavelengths 31.2 -> 17.7 us, 512
+//    43.6 -> 17.3, two lines 64 -> 23; 150 models of 512 wavelengths 46 -> 37,
+//    but 600 107 against 128 (every block builds the model's tables).
+inline int blocks_per_model64(int n, int nl, int ncomp, int pass)
+{
+    if (n >= 2000 && nl <= (ncomp > 40 ? 6 : 12)) return 0;
+    return n <= kSMs ? (nl + pass - 1) / pass : 1;
+}
+
 }  // namespace genesis

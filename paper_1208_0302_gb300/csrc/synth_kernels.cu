@@ -251,9 +251,10 @@ k_vjp(const __grid_constant__ KProblem pb, const double *__restrict__ params,
     }
 }
 
-// FP64 synthesis, one block per model (see profiles64.cuh): 65 536 two-line
-// models 14.0 -> 4.8 ms against a thread per (model, wavelength), a call for one
-// one-line model 27 -> 12.5 us; absolute error 1.5e-15 -> 7e-17 rms.
+// FP64 synthesis, one block per model (see profiles64.cuh), or one per pass over
+// its wavelengths (blocks_per_model64): 65 536 two-line models 14.0 -> 4.8 ms
+// against a thread per (model, wavelength) with Weideman's series, a call for
+// one one-line model 27 -> 12.5 us; absolute error 1.5e-15 -> 7e-17 rms.
 template <bool FILL>
 __global__ void __launch_bounds__(kProfBlock)
 k_synth64(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
@@ -537,11 +538,13 @@ template <bool FILL>
 cudaError_t synth64_t(const KProblem &pb, const double *params, const double *mu_px, int n, void *stokes,
                       cudaStream_t st)
 {
+    const int blocks = blocks_per_model64(n, pb.n_lambda, prof_components(pb), kProfBlock);
+    if (blocks == 0) return points_t<double, 0, FILL, false>(pb, params, mu_px, n, stokes, nullptr, st);
     auto kern = k_synth64<FILL>;
     const size_t smem = prof_smem(pb);
     cudaError_t e = allow_smem(kern, smem);
     if (e != cudaSuccess) return e;
-    kern<<<n, kProfBlock, smem, st>>>(pb, params, mu_px, (double *)stokes);
+    kern<<<dim3(n, blocks), kProfBlock, smem, st>>>(pb, params, mu_px, (double *)stokes);
     return cudaGetLastError();
 }
 

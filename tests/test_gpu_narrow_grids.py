@@ -46,3 +46,21 @@ def test_fp32_points(gpu, orc, kind, nl, n, fill):
     scale = want.abs().amax(dim=(1, 2), keepdim=True) + 1e-30
     err, ref = (torch.max((j.double() - want).abs() / scale).item() for j in (jac[:len(P)], general))
     assert err < 2 * ref + 1e-6, (err, ref)
+
+
+@pytest.mark.parametrize("kind,nl,n,fill", [("one", 3, 2001, False), ("two", 12, 2500, False), ("heavy", 6, 2000, False),
+                                            ("two", 8, 3001, True),                       # a thread per point
+                                            ("one", 129, 152, False), ("pattern", 300, 5, True),  # a block per pass
+                                            ("two", 512, 1, False), ("two", 257, 153, False)])
+def test_fp64_shapes(gpu, orc, kind, nl, n, fill):
+    spec, P = _spec(kind, nl, fill), _params(fill, nl)
+    P[:3, 5] = [0.0, 10.05, -0.0]  # none, beyond the node grid, none
+    P[3, 4] = 0.5                  # narrow lines: |x| to thousands
+    pb = gpu.Problem.from_spec(spec, "f64")
+    rows = torch.arange(n, device="cuda") % len(P)
+    got = gpu.me_synth(pb, torch.tensor(P, device="cuda")[rows].contiguous())
+    m = min(n, len(P))
+    assert torch.equal(got, got[:m][rows])
+    ref = orc.synth(spec, P[:m])
+    ic = (P[:m, 7] + P[:m, 8])[:, None, None]
+    assert np.max(np.abs(got[:m].cpu().numpy() - ref) / np.maximum(np.abs(ref), ic)) <= 1e-12

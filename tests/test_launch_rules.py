@@ -20,6 +20,10 @@ int main()
             int jac, lines, ncomp, triplets, nl, n;
             if (std::scanf("%d %d %d %d %d %d", &jac, &lines, &ncomp, &triplets, &nl, &n) != 6) return 1;
             std::printf("%d\n", chunks_per_warp(jac, n, nl, lines, ncomp, triplets, jac ? 4 : 8));
+        } else if (!std::strcmp(rule, "blocks64")) {
+            int n, nl, ncomp;
+            if (std::scanf("%d %d %d", &n, &nl, &ncomp) != 3) return 1;
+            std::printf("%d\n", blocks_per_model64(n, nl, ncomp, 128));
         }
     }
 }
@@ -60,3 +64,19 @@ def test_models_or_points(rule):
     for (case, points, models), (per,) in zip(MODELS, rule([("models",) + m[0] for m in MODELS])):
         assert (per == 0) == (points < models), (case, per)
         assert per <= (case[4] + 31) // 32
+
+
+# (models, wavelengths, components): us of k_points, of a block per model, of a block per pass
+BLOCKS64 = [((20000, 3, 3), 66.2, 325.5, None), ((20000, 8, 6), 245.2, 424.6, None), ((20000, 8, 15), 539.6, 856.0, None),
+            ((20000, 6, 69), 1797.0, 2801.9, None), ((20000, 24, 6), 675.8, 504.6, None), ((20000, 24, 69), 6346.8, 4116.0, None),
+            ((600, 8, 3), 20.9, 16.5, None), ((2500, 32, 6), 138.7, 86.9, None), ((1, 257, 3), 18.9, 31.2, 17.7),
+            ((1, 512, 6), 33.5, 64.3, 23.1), ((20, 512, 69), 203.6, 535.8, 145.4), ((150, 384, 15), 144.3, 99.6, 72.9),
+            ((600, 512, 6), 319.6, 163.6, 183.7), ((20000, 257, 3), 3041.5, 1968.8, 2486.2), ((1, 64, 3), 19.0, 13.1, 13.1)]
+
+
+def test_blocks_per_fp64_model(rule):
+    for (case, points, one, passes), (got,) in zip(BLOCKS64, rule([("blocks64",) + b[0] for b in BLOCKS64])):
+        best = min(t for t in (points, one, passes) if t is not None)
+        took = {0: points, 1: one}.get(got, passes)
+        assert took <= best * 1.06, (case, got)
+        assert got <= (case[1] + 127) // 128
