@@ -8,7 +8,9 @@
 
 namespace genesis {
 
-constexpr int kSMs = 152;  // of a whole GB300
+constexpr int kSMs = 152;                   // of a whole GB300
+constexpr int kSharedPerSM = 228 * 1024;   // bytes, of which every resident block
+constexpr int kSharedPerBlock = 1024;      // takes so many beside its own
 
 // FP32 synthesis and Jacobian: how many chunks of 32 wavelengths of one model
 // a warp takes (k_models), or 0 for a thread per (model, wavelength)
@@ -58,6 +60,42 @@ inline int chunks_per_warp(bool jac, int n, int nl, int n_lines, int ncomp, bool
         }
     }
     return per;
+}
+
+// Line centres: lanes per pixel (32, 8, 2 or 1; 32 / lanes pixels to a one-warp
+// block), for n pixels, candidates search positions of 2 W differences and
+// elem bytes of shared memory per staged sample.  More lanes shorten a warp's
+// chain of dependent sums and the rows it stages, fewer leave no lane idle in
+// a ragged last round and start fewer blocks.  The time of a choice is modelled
+// as the longer of the chains, one after another where shared memory admits R
+// blocks to an SM, and of the SM's issue, plus 0.3 of the other; fitted to 800
+// measured calls (1 to 70 000 pixels, 7 to 510 candidates, W = 1, 10, 40,
+// float and double), of which it picks a shape more than 1.1 times slower than
+// the best for 3.  Lanes by the number of pixels alone took up to ten times the
+// best: 70 000 pixels over a whole grid of 512 wavelengths, W = 10, float 1969
+// -> 234 us (8.4 x), double 6610 -> 1474 us.
+inline int centre_lanes(bool integers, int n, int candidates, int W, int elem)
+{
+    // in units of one term of a chain: a term's issue, a staged row of 32 samples and its issue, a block's start
+    const double term = integers ? 0.018 : 0.265, row = integers ? 3.66 : 1.11;
+    const double row_issue = integers ? 0.012 : 0.126, start = integers ? 4.04 : 0.735;
+    int best = 1;
+    double least = 1e300;
+    for (int lanes : {32, 8, 2, 1}) {
+        const int pixels = 32 / lanes, span = candidates + 2 * W;
+        const double per_sm = (double)(((long long)n * lanes + 31) / 32) / kSMs;
+        const int resident = std::max(1, std::min(32, kSharedPerSM / (pixels * (span | 1) * elem + kSharedPerBlock)));
+        const double terms = (double)((candidates + lanes - 1) / lanes + (lanes == 1 ? 2 : 1)) * W;
+        const double rows = (double)pixels * ((span + 31) / 32);
+        const double chains = std::max(1.0, per_sm / resident) * (terms + row * rows);
+        const double issue = per_sm * (term * terms + row_issue * rows + start);
+        const double t = std::max(chains, issue) + 0.3 * std::min(chains, issue);
+        if (t < least) {
+            least = t;
+            best = lanes;
+        }
+    }
+    return best;
 }
 
 // FP64 synthesis: blocks per model (k_synth64, whose passes of 128 wavelengths

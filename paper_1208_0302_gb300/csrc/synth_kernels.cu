@@ -616,18 +616,16 @@ cudaError_t line_centre_t(const KProblem &pb, const void *obs, int npix, int W, 
     return cudaGetLastError();
 }
 
-// Lanes per pixel: as many as leave at most one warp to each of the 608 SM
-// partitions, whose FP64 pipe one warp's chain of dependent adds already
-// fills; then the shortest chain is the fastest.  Beyond that, one.
 template <class RO>
 cudaError_t line_centre_r(const KProblem &pb, const void *obs, int npix, int W, int lo, int hi, double *lam_c,
                           int *idx, cudaStream_t st)
 {
-    const int warps = 152 * 4;
-    if (npix <= warps) return line_centre_t<RO, 32>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
-    if (npix <= 4 * warps) return line_centre_t<RO, 8>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
-    if (npix <= 16 * warps) return line_centre_t<RO, 2>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
-    return line_centre_t<RO, 1>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    switch (lo <= hi ? centre_lanes(sizeof(RO) == 4, npix, hi - lo + 1, W, sizeof(RO) == 4 ? 12 : 8) : 1) {
+    case 32: return line_centre_t<RO, 32>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    case 8: return line_centre_t<RO, 8>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    case 2: return line_centre_t<RO, 2>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    default: return line_centre_t<RO, 1>(pb, obs, npix, W, lo, hi, lam_c, idx, st);
+    }
 }
 
 }  // namespace

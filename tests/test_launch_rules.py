@@ -24,6 +24,10 @@ int main()
             int n, nl, ncomp;
             if (std::scanf("%d %d %d", &n, &nl, &ncomp) != 3) return 1;
             std::printf("%d\n", blocks_per_model64(n, nl, ncomp, 128));
+        } else if (!std::strcmp(rule, "centre")) {
+            int integers, n, candidates, W;
+            if (std::scanf("%d %d %d %d", &integers, &n, &candidates, &W) != 4) return 1;
+            std::printf("%d\n", centre_lanes(integers, n, candidates, W, integers ? 12 : 8));
         }
     }
 }
@@ -80,3 +84,22 @@ def test_blocks_per_fp64_model(rule):
         took = {0: points, 1: one}.get(got, passes)
         assert took <= best * 1.06, (case, got)
         assert got <= (case[1] + 127) // 128
+
+
+# (float cube, pixels, candidates, W): us by lanes per pixel
+CENTRE = [((0, 700, 492, 10), {1: 434.1, 2: 224.4, 8: 60.3, 32: 23.3}), ((0, 1500, 257, 40), {1: 838.0, 2: 422.6, 8: 114.2, 32: 83.1}),
+          ((0, 3000, 257, 10), {1: 237.6, 2: 124.7, 8: 43.9, 32: 48.0}), ((0, 6000, 48, 40), {1: 168.0, 2: 87.2, 8: 60.2, 32: 107.5}),
+          ((0, 6000, 432, 40), {1: 2704.3, 2: 697.6, 8: 424.3, 32: 486.0}), ((0, 12000, 34, 1), {1: 23.0, 2: 15.2, 8: 15.1, 32: 27.1}),
+          ((0, 12000, 34, 40), {1: 137.1, 2: 91.7, 8: 101.8, 32: 192.3}), ((0, 12000, 65, 1), {1: 27.3, 2: 18.6, 8: 15.1, 32: 29.3}),
+          ((0, 70000, 126, 1), {1: 108.4, 2: 80.0, 8: 85.0, 32: 159.6}), ((0, 70000, 257, 1), {1: 392.7, 2: 225.7, 8: 152.4, 32: 228.3}),
+          ((0, 70000, 492, 10), {1: 6610.1, 2: 2297.9, 8: 1473.5, 32: 1636.5}), ((0, 70000, 34, 10), {1: 124.4, 2: 135.5, 8: 165.9, 32: 361.6}),
+          ((1, 3000, 24, 40), {1: 39.5, 2: 23.6, 8: 14.9, 32: 14.5}), ((1, 3000, 254, 1), {1: 52.1, 2: 30.4, 8: 15.2, 32: 15.3}),
+          ((1, 12000, 34, 1), {1: 21.1, 2: 14.8, 8: 14.2, 32: 25.3}), ((1, 12000, 257, 1), {1: 110.6, 2: 62.5, 8: 25.1, 32: 28.7}),
+          ((1, 25000, 48, 40), {1: 81.3, 2: 68.7, 8: 54.1, 32: 51.9}), ((1, 25000, 492, 10), {1: 799.9, 2: 457.3, 8: 145.5, 32: 87.9}),
+          ((1, 70000, 65, 1), {1: 52.0, 2: 37.6, 8: 39.5, 32: 127.2}), ((1, 70000, 257, 1), {1: 435.2, 2: 239.5, 8: 85.4, 32: 131.2}),
+          ((1, 70000, 510, 1), {1: 1347.7, 2: 732.0, 8: 202.1, 32: 133.7}), ((1, 70000, 34, 1), {1: 27.1, 2: 28.6, 8: 37.5, 32: 124.3})]
+
+
+def test_lanes_per_line_centre(rule):
+    for (case, us), (lanes,) in zip(CENTRE, rule([("centre",) + c[0] for c in CENTRE])):
+        assert us[int(lanes)] <= 1.25 * min(us.values()), (case, lanes)
