@@ -16,6 +16,7 @@
 
 #include "fitness64.cuh"
 #include "kernels.h"
+#include "launch_rules.h"
 #include "me_pair.cuh"
 #include "rng_device.cuh"
 
@@ -585,13 +586,15 @@ __device__ __forceinline__ void weight_obs_rows(R *s_obs, int nl, int k, const R
 #endif
 // Build option: GENESIS_GA_MAXNREG=N caps every instantiation at N registers
 // per thread instead (for tuning the cap).
+constexpr int ga_registers(int maxt, int elem, int nl, bool pat, bool split)
+{
 #ifdef GENESIS_GA_MAXNREG
-#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT) __maxnreg__(GENESIS_GA_MAXNREG)
+    return GENESIS_GA_MAXNREG;
 #else
-#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT)                                                  \
-    __maxnreg__((MAXT) > 256 ? 65536 / (MAXT)                                                     \
-                             : (sizeof(R) == 4 ? ((NL) > 0 && !(PAT) ? GENESIS_GA_NREG32 : 80) : (SPLIT) ? 128 : 255))
+    return maxt > 256 ? 65536 / maxt : elem == 4 ? (nl > 0 && !pat ? GENESIS_GA_NREG32 : 80) : split ? 128 : 255;
 #endif
+}
+#define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT) __maxnreg__(ga_registers(MAXT, sizeof(R), NL, PAT, SPLIT))
 
 // SPLIT: blockDim.x / npop threads per individual share its wavelengths (FP32:
 // pairs; FP64: the shares of fitness64.cuh).  With fewer pixels than fill the chip at a block of npop threads
@@ -794,25 +797,6 @@ k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,
     }
 }
 
-// Threads per individual for npix pixels: as many as keep an SM's share of
-// the pixels within the warps its registers hold (FP32: 28 at 72 registers,
-// 24 at 80; FP64: 16 at 128); 1 = no split.  FP64 takes a power of two, so
-// that the shares divide evenly.  A split block does more work for the same
-// pixels (each segment forms the geometry, one breeds), which only costs where
-// `others`, the warps that other launches bring meanwhile, fill the GPU twice
-// over: a burst of 24 serving requests took 325 ms with each split as if it
-// ran alone and takes 300 ms with this rule, while four requests that just
-// fill the GPU take 24 ms split, 28 ms unsplit and 48 ms with the first alone
-// split.
-inline int ga_segments(int npix, int npop, int nl, int regs, long long others)
-{
-    if (others >= 2ll * 28 * 152) return 1;
-    const int warps = regs <= 72 ? 28 : regs <= 80 ? 24 : 16, per_sm = (npix + 151) / 152;
-    const int s = warps / (per_sm * (npop / 32)), npair = (nl + 1) / 2;
-    if (regs > 80) return s >= 8 ? 8 : s >= 4 ? 4 : s >= 2 ? 2 : 1;
-    return s < npair ? s : npair;
-}
-
 template <class R, int NL, int MAXT, bool COUNT = false, bool PAT = false, int M = ME_NPAR>
 cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, const double *w,
                             const double *mu_px, int npix, double *best, uint16_t *best_genes,
@@ -821,9 +805,9 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
 {
     const int nlines = NL > 0 ? NL : pb.n_lines;
     if constexpr (MAXT <= 256 && !COUNT) {
-        const int regs = sizeof(R) == 8 ? 128 : NL > 0 && !PAT ? GENESIS_GA_NREG32 : 80;
-        const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, regs, others);
         const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M, true);
+        const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, ga_registers(MAXT, sizeof(R), NL, PAT, true), sizeof(R) == 8,
+                                     others);
         if (nseg > 1 && L.total <= 200 * 1024) {
             auto kern = k_ga_evolve<R, NL, MAXT, false, PAT, M, true>;
             cudaError_t e = allow_smem(kern, L.total);

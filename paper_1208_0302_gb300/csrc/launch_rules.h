@@ -9,8 +9,10 @@
 namespace genesis {
 
 constexpr int kSMs = 152;                   // of a whole GB300
-constexpr int kSharedPerSM = 228 * 1024;   // bytes, of which every resident block
-constexpr int kSharedPerBlock = 1024;      // takes so many beside its own
+
+// Blocks of so many bytes of shared memory that an SM's 228 KB hold: each takes
+// 1 KB beside its own, which come in steps of 256 bytes.
+inline int blocks_by_shared(int bytes) { return 228 * 1024 / ((bytes + 255) / 256 * 256 + 1024); }
 
 // FP32 synthesis and Jacobian: how many chunks of 32 wavelengths of one model
 // a warp takes (k_models), or 0 for a thread per (model, wavelength)
@@ -62,6 +64,32 @@ inline int chunks_per_warp(bool jac, int n, int nl, int n_lines, int ncomp, bool
     return per;
 }
 
+// Warps of a kernel of so many registers per thread that fit an SM, in steps of
+// four (one to each partition) and no more than a block can have.
+inline int resident_warps(int regs) { return std::min(32, 65536 / ((regs + 7) / 8 * 8 * 32)) / 4 * 4; }
+
+// GA: threads per individual (segments) for npix pixels; 1 = no split.
+//  * As many as keep an SM's share of the pixels within the warps its
+//    registers hold: with few pixels an SM holds only a few warps and the
+//    fitness loop is a chain of dependent operations.  FP64 takes a power of
+//    two, so that the eight shares of an individual's wavelengths divide
+//    evenly.
+//  * A split block does more work for the same pixels (each segment forms the
+//    geometry, one breeds), which only costs where `others`, the warps that
+//    other launches bring meanwhile, fill the GPU twice over: a burst of 24
+//    serving requests took 325 ms with each split as if it ran alone and takes
+//    300 ms with this rule, while four requests that just fill the GPU take 24
+//    ms split, 28 ms unsplit and 48 ms with the first alone split.
+inline int ga_segments(int npix, int npop, int nl, int regs, bool fp64, long long others)
+{
+    const int room = resident_warps(regs), per_sm = (npix + kSMs - 1) / kSMs, each = npop / 32;
+    if (others >= 2ll * 28 * kSMs) return 1;
+    int s = room / (per_sm * each);
+    if (fp64) return s >= 8 ? 8 : s >= 4 ? 4 : s >= 2 ? 2 : 1;
+    const int npair = (nl + 1) / 2;
+    return s < npair ? s : npair;
+}
+
 // Line centres: lanes per pixel (32, 8, 2 or 1; 32 / lanes pixels to a one-warp
 // block), for n pixels, candidates search positions of 2 W differences and
 // elem bytes of shared memory per staged sample.  More lanes shorten a warp's
@@ -84,7 +112,7 @@ inline int centre_lanes(bool integers, int n, int candidates, int W, int elem)
     for (int lanes : {32, 8, 2, 1}) {
         const int pixels = 32 / lanes, span = candidates + 2 * W;
         const double per_sm = (double)(((long long)n * lanes + 31) / 32) / kSMs;
-        const int resident = std::max(1, std::min(32, kSharedPerSM / (pixels * (span | 1) * elem + kSharedPerBlock)));
+        const int resident = std::max(1, std::min(32, blocks_by_shared(pixels * (span | 1) * elem)));
         const double terms = (double)((candidates + lanes - 1) / lanes + (lanes == 1 ? 2 : 1)) * W;
         const double rows = (double)pixels * ((span + 31) / 32);
         const double chains = std::max(1.0, per_sm / resident) * (terms + row * rows);

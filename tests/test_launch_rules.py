@@ -24,6 +24,15 @@ int main()
             int n, nl, ncomp;
             if (std::scanf("%d %d %d", &n, &nl, &ncomp) != 3) return 1;
             std::printf("%d\n", blocks_per_model64(n, nl, ncomp, 128));
+        } else if (!std::strcmp(rule, "segments")) {
+            int npix, npop, nl, regs, fp64;
+            long long others;
+            if (std::scanf("%d %d %d %d %d %lld", &npix, &npop, &nl, &regs, &fp64, &others) != 6) return 1;
+            std::printf("%d\n", ga_segments(npix, npop, nl, regs, fp64, others));
+        } else if (!std::strcmp(rule, "warps")) {
+            int regs;
+            if (std::scanf("%d", &regs) != 1) return 1;
+            std::printf("%d\n", resident_warps(regs));
         } else if (!std::strcmp(rule, "centre")) {
             int integers, n, candidates, W;
             if (std::scanf("%d %d %d %d", &integers, &n, &candidates, &W) != 4) return 1;
@@ -103,3 +112,15 @@ CENTRE = [((0, 700, 492, 10), {1: 434.1, 2: 224.4, 8: 60.3, 32: 23.3}), ((0, 150
 def test_lanes_per_line_centre(rule):
     for (case, us), (lanes,) in zip(CENTRE, rule([("centre",) + c[0] for c in CENTRE])):
         assert us[int(lanes)] <= 1.25 * min(us.values()), (case, lanes)
+
+
+def test_split_blocks_fit_the_registers(rule):
+    """A split block is launchable whatever cap the kernels are built with."""
+    regs = list(range(24, 256))
+    for r, (warps,) in zip(regs, rule([("warps", r) for r in regs])):
+        assert 4 <= warps <= 32 and warps * 32 * -(-r // 8) * 8 <= 65536
+    for npop in (32, 64, 96, 128, 256):
+        calls = [("segments", n, npop, 128, r, fp64, 0) for n in (1, 152, 153, 500) for r in regs for fp64 in (0, 1)]
+        for c, (s,) in zip(calls, rule(calls)):
+            assert s == 1 or s * npop * -(-c[4] // 8) * 8 <= 65536, c
+            assert s * npop <= 1024
