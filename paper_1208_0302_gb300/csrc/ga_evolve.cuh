@@ -807,7 +807,7 @@ cudaError_t launch_evolve_t(const KProblem &pb, const KGa &ga, const void *obs, 
     if constexpr (MAXT <= 256 && !COUNT) {
         const GaSmem L = ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M, true);
         const int nseg = ga_segments(npix, ga.npop, pb.n_lambda, ga_registers(MAXT, sizeof(R), NL, PAT, true), sizeof(R) == 8,
-                                     others);
+                                     L.total, ga_smem_layout<R>(pb.n_lambda, nlines, ga.npop, M).total, others);
         if (nseg > 1 && L.total <= 200 * 1024) {
             auto kern = k_ga_evolve<R, NL, MAXT, false, PAT, M, true>;
             cudaError_t e = allow_smem(kern, L.total);

@@ -80,14 +80,39 @@ inline int resident_warps(int regs) { return std::min(32, 65536 / ((regs + 7) / 
 //    serving requests took 325 ms with each split as if it ran alone and takes
 //    300 ms with this rule, while four requests that just fill the GPU take 24
 //    ms split, 28 ms unsplit and 48 ms with the first alone split.
-inline int ga_segments(int npix, int npop, int nl, int regs, bool fp64, long long others)
+//  * An FP32 split block also holds a float per pair of wavelengths and
+//    individual, so on wide grids fewer blocks fit an SM and the pixels take
+//    turns.  A round of w resident warps, rounded up to the four partitions of
+//    an SM, takes max(10, w + 4) units for a warp's work (two lines, population
+//    128, 256 wavelengths, 1 to 7 blocks to an SM: 952, 1161, 1524, 1886, 2682
+//    and 3063 us at 4, 8, 12, 16, 24 and 28 warps); its work is its pairs and
+//    four more for what every segment does.  Where the split blocks do not all
+//    fit, the split runs if its rounds take less than those without: of 301
+//    measured sizes (111 to 512 wavelengths, populations 32 to 160, 1 to 14
+//    pixels to an SM) the slower side is picked by more than 5 % for 4, at most
+//    10 %.  Population 128, 456 pixels: 384 wavelengths 2606 us split, 2061
+//    not, 512 wavelengths 3414 and 2689; population 64: 1064 pixels, 192
+//    wavelengths 1296 and 1448, 608 pixels, 128 wavelengths 536 and 599.
+// shared_split, shared_plain: bytes of a block with and without the split.
+inline int ga_segments(int npix, int npop, int nl, int regs, bool fp64, int shared_split, int shared_plain,
+                       long long others)
 {
     const int room = resident_warps(regs), per_sm = (npix + kSMs - 1) / kSMs, each = npop / 32;
     if (others >= 2ll * 28 * kSMs) return 1;
     int s = room / (per_sm * each);
     if (fp64) return s >= 8 ? 8 : s >= 4 ? 4 : s >= 2 ? 2 : 1;
     const int npair = (nl + 1) / 2;
-    return s < npair ? s : npair;
+    s = std::min(s, npair);
+    if (s < 2) return 1;
+    auto fit = [&](int warps, int shared) { return std::max(1, std::min(room / warps, blocks_by_shared(shared))); };
+    if (per_sm <= fit(s * each, shared_split)) return s;  // no turns
+    auto rounds = [&](int warps, int shared) -> long long {
+        const int f = fit(warps, shared), rest = per_sm % f;
+        auto round = [](int w) { return w ? std::max(10, (w + 3) / 4 * 4 + 4) : 0; };
+        return per_sm / f * round(f * warps) + round(rest * warps);
+    };
+    const long long split = rounds(s * each, shared_split) * ((npair + s - 1) / s + 4);
+    return split < rounds(each, shared_plain) * (npair + 4) ? s : 1;
 }
 
 // Line centres: lanes per pixel (32, 8, 2 or 1; 32 / lanes pixels to a one-warp

@@ -25,10 +25,10 @@ int main()
             if (std::scanf("%d %d %d", &n, &nl, &ncomp) != 3) return 1;
             std::printf("%d\n", blocks_per_model64(n, nl, ncomp, 128));
         } else if (!std::strcmp(rule, "segments")) {
-            int npix, npop, nl, regs, fp64;
+            int npix, npop, nl, regs, fp64, split, plain;
             long long others;
-            if (std::scanf("%d %d %d %d %d %lld", &npix, &npop, &nl, &regs, &fp64, &others) != 6) return 1;
-            std::printf("%d\n", ga_segments(npix, npop, nl, regs, fp64, others));
+            if (std::scanf("%d %d %d %d %d %d %d %lld", &npix, &npop, &nl, &regs, &fp64, &split, &plain, &others) != 8) return 1;
+            std::printf("%d\n", ga_segments(npix, npop, nl, regs, fp64, split, plain, others));
         } else if (!std::strcmp(rule, "warps")) {
             int regs;
             if (std::scanf("%d", &regs) != 1) return 1;
@@ -114,13 +114,39 @@ def test_lanes_per_line_centre(rule):
         assert us[int(lanes)] <= 1.25 * min(us.values()), (case, lanes)
 
 
+def ga_shared(nl, npop, split):
+    """Bytes of an FP32 GA block with nine parameters (ga_smem_layout)."""
+    pairs, total = (nl + 1) // 2, 0
+    for n in (32 * pairs, 32 * pairs, 4 * npop, 128, 128, 32, 16, 240, 2048, 36 * npop, 64 * npop, 4 * pairs * npop * split):
+        total = -(-total // 16) * 16 + n
+    return -(-total // 16) * 16
+
+
+# (pixels, population, wavelengths, registers): us split, us unsplit
+SEGMENTS = [((456, 128, 384, 72), 2606, 2061), ((304, 128, 384, 80), 4475, 5505), ((456, 128, 512, 72), 3414, 2689),
+            ((912, 64, 512, 72), 3448, 2867), ((1520, 32, 512, 72), 3500, 4335), ((608, 64, 128, 72), 536, 599),
+            ((64, 64, 128, 72), 538, 1800), ((1, 128, 256, 72), 466, 930), ((304, 64, 256, 72), 508, 997)]
+
+
+def test_ga_split(rule):
+    calls = [("segments",) + c + (0, ga_shared(c[2], c[1], 1), ga_shared(c[2], c[1], 0), 0) for c, _, _ in SEGMENTS]
+    for (case, split, plain), (n,) in zip(SEGMENTS, rule(calls)):
+        assert (n > 1) == (split < plain), (case, n)
+    # up to 144 wavelengths as many segments as the registers hold, but for a block or two to an SM
+    (few,), (many,), (fp64,), (busy,) = rule([("segments", 64, 64, 128, 72, 0, ga_shared(128, 64, 1), ga_shared(128, 64, 0), 0),
+                                              ("segments", 20000, 64, 128, 72, 0, ga_shared(128, 64, 1), ga_shared(128, 64, 0), 0),
+                                              ("segments", 256, 64, 64, 128, 1, 60000, 60000, 0),
+                                              ("segments", 64, 64, 128, 72, 0, ga_shared(128, 64, 1), ga_shared(128, 64, 0), 8512)])
+    assert (few, many, fp64, busy) == (14, 1, 4, 1)
+
+
 def test_split_blocks_fit_the_registers(rule):
     """A split block is launchable whatever cap the kernels are built with."""
     regs = list(range(24, 256))
     for r, (warps,) in zip(regs, rule([("warps", r) for r in regs])):
         assert 4 <= warps <= 32 and warps * 32 * -(-r // 8) * 8 <= 65536
     for npop in (32, 64, 96, 128, 256):
-        calls = [("segments", n, npop, 128, r, fp64, 0) for n in (1, 152, 153, 500) for r in regs for fp64 in (0, 1)]
+        calls = [("segments", n, npop, 128, r, fp64, 10000, 9000, 0) for n in (1, 152, 153, 500) for r in regs for fp64 in (0, 1)]
         for c, (s,) in zip(calls, rule(calls)):
             assert s == 1 or s * npop * -(-c[4] // 8) * 8 <= 65536, c
             assert s * npop <= 1024
