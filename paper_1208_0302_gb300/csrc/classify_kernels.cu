@@ -3,6 +3,7 @@
 #include "async_copy.cuh"
 #include "fp64_util.cuh"
 #include "kernels.h"
+#include "launch_rules.h"
 
 namespace genesis {
 
@@ -495,7 +496,7 @@ cudaError_t launch_classify(const KProblem &pb, int dtype, const void *obs, int 
                             cudaStream_t st)
 {
     if (npix <= 0) return cudaSuccess;
-    const bool chain = npix <= 152 * 4 / 2 * 32;
+    const bool chain = npix <= kSMs * 4 / 2 * 32;
     if (dtype == ME_F32) return chain ? classify_t<float, 2>(pb, obs, npix, c, st) : classify_t<float, 1>(pb, obs, npix, c, st);
     return chain ? classify_t<double, 2>(pb, obs, npix, c, st) : classify_t<double, 1>(pb, obs, npix, c, st);
 }
