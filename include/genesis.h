@@ -170,6 +170,11 @@ int me_version(void);
  *   mu_px   dev double [n] or NULL (then pb->mu)
  *   stokes  dev [n][4][n_lambda] of pb->dtype (output)
  * n = 0 is a no-op.
+ * FP64: here and in me_chi2 w(z) comes from Taylor expansions and convergents
+ * (absolute error of the profiles 2e-16); me_synth_jac, me_synth_vjp and the
+ * L-M take Weideman's series (2e-15), so their Stokes differ by about 1e-15.
+ * Dampings below 0 are not physical; w(z) is continued to them, to full
+ * accuracy down to -1 and not at all below -2.
  */
 int me_synth(const me_problem *pb, const double *params, const double *mu_px, int n,
              void *stokes, void *stream);
@@ -244,8 +249,12 @@ int ga_count_evaluations(const me_problem *pb, const void *obs, const double *w,
  * ga_fitness - the fitness that ga_invert_batch ranks its population by, for
  * caller-given individuals: Eq. chisq of the Section 5 synthesis, in
  * pb->dtype arithmetic (FP32: the packed two-wavelength pair path with its
- * warp-voted w(z) regions; FP64: the per-wavelength path), with the GA's
- * launch shape and the kernel instantiation ga_invert_batch would choose.
+ * warp-voted w(z) regions; FP64: w(z) from the node grid and the convergents
+ * and eight compensated sums over the wavelengths up to npop 256, Weideman's
+ * series and a compensated sum per Stokes parameter above), evaluated as
+ * ga_invert_batch evaluates it with one thread per individual.  (With few
+ * pixels ga_invert_batch shares an individual's wavelengths among threads;
+ * the values are the same bits.)
  * One thread block per pixel and one thread per individual; only threads
  * k < nactive evaluate, inside a divergent branch as the GA's restarts do
  * (nactive = npop / 2 = 16 of npop = 32 is the restart of the smallest

@@ -2,14 +2,15 @@
 // Algorithm 1; Section 5.6), shared by the translation units that instantiate
 // it (9 parameters; 10 with the fill fraction of Section 5.2).
 //
-//
-// One thread block per pixel, one thread per individual.  The pixel's
+// One thread block per pixel; one thread per individual, or, with few pixels,
+// several that share the individual's wavelengths (see SPLIT).  The pixel's
 // observed Stokes profiles, its wavelength offsets, the population's uint16
 // genotypes (double-buffered) and fitness stay in shared memory for all
 // generations; no host round trip happens between generations.  Each thread
-// walks the wavelength grid for its own individual, so every lane of a warp
-// reads the same shared-memory word (broadcast) and the chi2 sum needs no
-// cross-thread reduction.
+// walks the wavelength grid, or its share of it, for its own individual, so
+// every lane of a warp reads the same shared-memory word (broadcast) and the
+// chi2 sum is formed by one thread, from the shares in a fixed order where it
+// is split.
 #pragma once
 
 #include <type_traits>
@@ -127,23 +128,11 @@ __device__ __forceinline__ R fitness_rows(const KProblem &pb, int nlines, int nl
 }
 
 
-// Eq. chisq for one individual with the FP32 pair path (two wavelengths per
-// step, packed FP32x2 arithmetic), as a Kahan-compensated sum.  The residuals
-// come out weighted: the staged Q, U, V rows carry the pixel's weights
-// (weight_obs_rows) and so do the individual's Q, U, V output constants, and
-// the I residual takes w_I with one multiply.  Each pair's eight squared
-// weighted residuals are summed by packed FMAs, its two lanes added, and the
-// result taken into one scalar running total with Kahan's compensation, so
-// the sum's relative error stays at a few units of 2^-24 whatever the number
-// of wavelengths.  The fitness only ranks
-// individuals; the best individual's chi2 is re-evaluated in FP64.
-// s_kc: the calling thread's shared-memory slots, three float4 at s_kc[k],
-// s_kc[k + blockDim], s_kc[k + 2 blockDim] (k = threadIdx.x), which hold the
-// individual's closed-form constants and w_I for the length of the call:
-// they are read once per pair instead of holding registers through the
-// profile evaluations.
 // The individual's geometry for the pair loop, its weights folded in and its
-// slots filled (k = its index, nt = the slots' stride).
+// slots filled (k = its index, nt = the slots' stride; see fitness_pairs).  In
+// a split block every segment fills them: the same code on the same inputs, so
+// the words that meet are the same bits, and a thread reads back only what it
+// or its equals wrote; no barrier is needed.
 template <int NL, bool FILL>
 __device__ __forceinline__ Geo<float> pair_geometry(const KProblem &pb, int nlines, const float *p, float mu,
                                                     const float *s_w2, float4 *s_kc, int k, int nt)
@@ -212,6 +201,21 @@ __device__ __forceinline__ void kahan_add(float &sum, float &comp, float v)
     sum = t;
 }
 
+// Eq. chisq for one individual with the FP32 pair path (two wavelengths per
+// step, packed FP32x2 arithmetic), as a Kahan-compensated sum.  The residuals
+// come out weighted: the staged Q, U, V rows carry the pixel's weights
+// (weight_obs_rows) and so do the individual's Q, U, V output constants, and
+// the I residual takes w_I with one multiply.  Each pair's eight squared
+// weighted residuals are summed by packed FMAs, its two lanes added, and the
+// result taken into one scalar running total with Kahan's compensation, so
+// the sum's relative error stays at a few units of 2^-24 whatever the number
+// of wavelengths.  The fitness only ranks
+// individuals; the best individual's chi2 is re-evaluated in FP64.
+// s_kc: the calling thread's shared-memory slots, three float4 at s_kc[k],
+// s_kc[k + blockDim], s_kc[k + 2 blockDim] (k = threadIdx.x), which hold the
+// individual's closed-form constants and w_I for the length of the call:
+// they are read once per pair instead of holding registers through the
+// profile evaluations.
 template <int NL, bool COUNT, bool PAT, bool FILL, bool STORE = false>
 __device__ __forceinline__ float fitness_pairs(const KProblem &pb, int nlines, int nl, const float *p,
                                                float mu, const float *s_obs, const float *s_doff,
@@ -597,13 +601,14 @@ constexpr int ga_registers(int maxt, int elem, int nl, bool pat, bool split)
 #define GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT) __maxnreg__(ga_registers(MAXT, sizeof(R), NL, PAT, SPLIT))
 
 // SPLIT: blockDim.x / npop threads per individual share its wavelengths (FP32:
-// pairs; FP64: the shares of fitness64.cuh).  With fewer pixels than fill the chip at a block of npop threads
-// each, an SM holds only a few warps and the fitness loop is a chain of
-// dependent operations; the shares run side by side.  A pair is evaluated by
+// pairs; FP64: the shares of fitness64.cuh).  With fewer pixels than fill the
+// chip at a block of npop threads each, an SM holds only a few warps and the
+// fitness loop is a chain of dependent operations; the shares run side by side.  A pair is evaluated by
 // the same lanes of a warp as without the split (so its votes, and with them
 // its bits, are the same), and the pairs' sums are added in the same order by
 // one thread, so the result does not depend on the split.  64 pixels,
-// population 64, 100 generations: 4.25 -> 1.68 ms.
+// population 64, 100 generations: 4.25 -> 1.39 ms.  ga_segments (launch_rules.h)
+// says where it runs.
 template <class R, int NL, int MAXT, bool COUNT, bool PAT, int M, bool SPLIT>
 __global__ void GENESIS_GA_BOUNDS(MAXT, R, NL, PAT, SPLIT)
 k_ga_evolve(const __grid_constant__ KProblem pb, const __grid_constant__ KGa ga,

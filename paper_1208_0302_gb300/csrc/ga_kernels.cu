@@ -1,13 +1,6 @@
-// Fused genetic-algorithm inversion kernel for sm_103a (Section 3, Algorithm 1;
-// Section 5.6), plus the operator-only kernels used to verify it.
-//
-// One thread block per pixel, one thread per individual.  The pixel's
-// observed Stokes profiles, its wavelength offsets, the population's uint16
-// genotypes (double-buffered) and fitness stay in shared memory for all
-// generations; no host round trip happens between generations.  Each thread
-// walks the wavelength grid for its own individual, so every lane of a warp
-// reads the same shared-memory word (broadcast) and the chi2 sum needs no
-// cross-thread reduction.
+// The 9-parameter instantiations of the fused genetic-algorithm kernel
+// (ga_evolve.cuh; Section 3, Algorithm 1; Section 5.6), and the operator-only
+// kernels used to verify it.
 #include "ga_evolve.cuh"
 
 namespace genesis {

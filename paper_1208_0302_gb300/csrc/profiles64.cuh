@@ -21,7 +21,7 @@
 //    1 / sqrt(pi), real polynomials whose coefficients depend on a^2 alone and
 //    are formed once per model): the 9th to |z|^2 = 170, the 7th to 500, the
 //    5th beyond, 23 to 35 operations where the 9th in complex arithmetic
-//    takes 56.  Each is within 3e-17 of w in its region.
+//    takes 56.  Each is within 4e-17 of w in its region.
 //  * Points of one region are gathered into lists, block-wide, so that every
 //    warp runs one branch with (nearly) all its lanes.
 #pragma once

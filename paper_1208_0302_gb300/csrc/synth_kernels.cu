@@ -75,7 +75,8 @@ constexpr int kJacMinB = 4;
 // and 32 wavelengths leaves through shared memory as 32 M consecutive values,
 // so that each store instruction writes whole sectors (lane by lane it wrote
 // 4 of every 36 bytes).  20 011 two-line FP32 models, 128 wavelengths:
-// syntheses 110 -> 55 us, Jacobians 267 -> 128 us.
+// syntheses 110 -> 55 us, Jacobians 267 -> 128 us.  chunks_per_warp says where
+// k_points is the faster one.
 template <int NL, bool FILL, bool JAC>
 __global__ void __launch_bounds__(kSynthBlock, JAC ? kJacMinB : 8)
 k_models(const __grid_constant__ KProblem pb, const double *__restrict__ params, const double *__restrict__ mu_px,
@@ -410,8 +411,8 @@ __device__ __forceinline__ void centre_search(const T *I, int W, int lo, int hi,
 // terms fit 53 bits, every difference and sum is exact in FP64 and equals the
 // same sum of 64-bit integers, which run on the integer pipe; other rows (and
 // double cubes) are summed in FP64.  262 144 pixels, W = 10, 33 candidates:
-// 2.40 ms with a warp per pixel in FP64, 0.47 ms with these lanes in FP64,
-// 0.15 ms with the integer sums.
+// 2.40 ms with a warp per pixel in FP64, 0.47 ms with a lane each in FP64, 0.15
+// ms with the integer sums, 0.12 ms with two lanes each (centre_lanes).
 template <class RO, int G>
 __global__ void __launch_bounds__(32)
 k_line_centre(const __grid_constant__ KProblem pb, const RO *__restrict__ obs, int npix, int W, int lo,
